@@ -8,8 +8,9 @@
 //
 // Schedules
 //  * k_plain  -- one thread per series runs the whole sequential filter
-//                (Eqs. integrated_kalman_pred/update, loglikelihood).  The FP64
-//                instantiation is the plain FP64 GPU baseline.
+//                (Eqs. integrated_kalman_pred/update, loglikelihood) in FP32.
+//                The plain FP64 filter is k_plain64 (gpss_plain64.cuh), two
+//                warps per series.
 //  * chunked parallel-in-time (Section 3.2.5, with the associative elements of
 //    Sarkka & Garcia-Fernandez 2021):
 //      k_elem     one thread per chunk of events; runs the filter from an
@@ -280,6 +281,12 @@ GPSS_D void flag_error(int *err, int row, int code) {
   if (err) atomicMax(err + row, code);
 }
 
+}  // namespace gpss
+
+#include "gpss_plain64.cuh"
+
+namespace gpss {
+
 // Asynchronous 16-byte global -> shared copy through L2 (cp.async.cg,
 // sm_80 and later), committed as groups; wait_group<N> returns once at most
 // N of this thread's groups are still in flight, and the thread then sees
@@ -391,12 +398,13 @@ GPSS_D const float4 *stage_table(const float *__restrict__ tab, int row, float4 
 }
 
 // ---------------------------------------------------------------------------
-// Plain per-series filter (loglik only).
+// Plain per-series filter (loglik only), FP32.
 // ---------------------------------------------------------------------------
-template <class S, class F>
+template <class S>
 __global__ void __launch_bounds__(128) k_plain(DevModel M, const float *__restrict__ theta, int n_out,
                                                int per_series, double *__restrict__ ll_out,
                                                int *__restrict__ err) {
+  using F = float;
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= n_out) return;
   const int s = per_series ? v : v % M.n_series;
@@ -463,7 +471,8 @@ GPSS_D void store_elem(float *dst, int n_vch, int vc, const float (&A)[S::D][S::
   }
 }
 
-// resident 128-thread blocks per SM the register budget of k_elem is sized for
+constexpr int ELEM_BS = 128;  // threads (chunks) per block of k_elem
+// resident blocks per SM the register budget of k_elem is sized for
 #ifndef GPSS_ELEM_MIN_BLOCKS
 #define GPSS_ELEM_MIN_BLOCKS 3
 #endif
@@ -555,7 +564,7 @@ GPSS_HD void elem_event(const Blocks<F> *B, uint8_t tag, F y, F r0, F w, F s2,
 // dcache set, every step's six scalars per term go to the step-scalar cache
 // (for the gradient's forward replay).
 template <class S, bool OD>
-__global__ void __launch_bounds__(128, ELEM_MIN_BLOCKS) k_elem(DevModel M, const float *__restrict__ theta, int n_vch,
+__global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, const float *__restrict__ theta, int n_vch,
                                               int per_series, float *__restrict__ ef,
                                               double *__restrict__ ed, int *__restrict__ err,
                                               const float *__restrict__ tabs,
@@ -1914,12 +1923,12 @@ struct OpTable {
 };
 
 
-template <class S, class F>
+template <class S>
 cudaError_t launch_plain(const DevModel &M, const float *theta, int n_out, int per_series,
                          double *ll, int *err, cudaStream_t st) {
   if (n_out <= 0) return cudaSuccess;
   const int bs = 128;
-  k_plain<S, F><<<(n_out + bs - 1) / bs, bs, 0, st>>>(M, theta, n_out, per_series, ll, err);
+  k_plain<S><<<(n_out + bs - 1) / bs, bs, 0, st>>>(M, theta, n_out, per_series, ll, err);
   GPSS_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -1931,7 +1940,7 @@ cudaError_t launch_elem(const DevModel &M, const float *theta, int n_vch, int pe
   if (n_vch <= 0 || c_count <= 0) return cudaSuccess;
   if (c_begin < 0 || c_begin + c_count > M.n_chunks) return cudaErrorInvalidValue;
   if (pck && (ck < 2 || ck > 64 || (ck & 1))) return cudaErrorInvalidValue;
-  const int bs = 128;
+  const int bs = ELEM_BS;
   const size_t smem = (size_t)(bs / 32) * S::NT * TAB_TERM * sizeof(float);
   // two launches: rows without an overdamped term (the lean body), then rows
   // with one; each skips the other's rows
@@ -2098,8 +2107,8 @@ OpTable make_ops() {
   o.NP = S::NP;
   o.NF = ElemLayout<S>::NF;
   o.ND = ElemLayout<S>::ND;
-  o.plain32 = &launch_plain<S, float>;
-  o.plain64 = &launch_plain<S, double>;
+  o.plain32 = &launch_plain<S>;
+  o.plain64 = &launch_plain64<S>;
   o.elem = &launch_elem<S>;
   o.grad = &launch_grad<S>;
   o.disc = &launch_disc<S>;
