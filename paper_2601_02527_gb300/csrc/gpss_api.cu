@@ -1614,10 +1614,17 @@ gp_ss_status gp_ss_loglik_grad_host(const gp_ss_model *m, const float *theta_hos
   // A re-sent event stream goes up in series groups on a second stream, and
   // each group's element pass starts as soon as its events are in (the copy
   // of the rest overlaps it).  The copy stream first waits for earlier work
-  // on st, which may still read the device copy.  Four groups (c4 element
-  // phase with the upload: 1.84 ms with four, 1.90 ms with two; 0.80 ms
-  // without the upload, 1.18 ms for the upload alone).
+  // on st, which may still read the device copy.  A group's element pass takes
+  // at least its longest chunk's serial time however few chunks it has, so a
+  // group is given at least one block of chunks per SM, and there are at most
+  // four groups (90112 chunks of two terms: element phase with the upload
+  // 1.84 ms with four, 1.90 ms with two; 11424 chunks: the whole call 1.75 ms
+  // with four, 1.17 ms with one).
   constexpr int kGroups = 4;
+  int n_sm = 0;
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, m->device);
+  const int n_groups =
+      std::max(1, std::min(kGroups, m->n_chunks / std::max(1, n_sm * gpss::ELEM_BS)));
   cudaStream_t cs = nullptr;
   cudaEvent_t start_ev = nullptr, ready[kGroups] = {};
   int c0[kGroups + 1] = {};
@@ -1627,8 +1634,8 @@ gp_ss_status gp_ss_loglik_grad_host(const gp_ss_model *m, const float *theta_hos
   float *d_meas3 = nullptr;
   if (pipe) {
     std::vector<int> sb{0};
-    for (int g = 1; g < kGroups; ++g) {
-      const int64_t target = m->ev_off[m->n_series] * g / kGroups;
+    for (int g = 1; g < n_groups; ++g) {
+      const int64_t target = m->ev_off[m->n_series] * g / n_groups;
       const int sp = (int)(std::lower_bound(m->ev_off.begin(), m->ev_off.end(), target) -
                            m->ev_off.begin());
       if (sp > sb.back() && sp < m->n_series) sb.push_back(sp);
