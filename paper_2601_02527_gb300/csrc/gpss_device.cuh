@@ -649,44 +649,118 @@ GPSS_HD Dual2<DF> operator*(Dual2<DF> x, DF c) { return mkdf(x.v * c, x.da * c, 
 // series j times T^(n + q_j) (q = 1 for f, f', F1; 2 for I_ff, I_pp, I_FF)
 // then follows from the c~ alone, and the economisation, linear with T fixed,
 // maps these to the table's coefficients times T^(k + q_j).
-// taylor_c_scaled: the recurrence into c (NCF + 1 entries).
-GPSS_HD void taylor_c_scaled(Dual2<DF> aT, Dual2<DF> w2T2, const DF *rcp, Dual2<DF> *c,
-                             DF T) {
-  const DF z = df_of(0.0);
-  c[0] = mkdf(z, z, z);
-  c[1] = mkdf(T, z, z);
-  c[2] = -(aT * T);
-  for (int n = 1; n + 2 <= TAB_NCF; ++n) {
-    const DF two_n1 = df_of(2.0 * (n + 1));
-    c[n + 2] = -((aT * two_n1) * c[n + 1] + w2T2 * c[n]) * (rcp[n + 2] * rcp[n + 1]);
-  }
+//
+// Tangents and the square of f' come from the structure of f instead of
+// forward-mode duals through every product (a third of the double-float
+// operations): with f = e^{-a t} sin(sqrt(beta) t)/sqrt(beta),
+//   df/da = -t f,          so  da c_n = -c_{n-1},
+//   g = df/dbeta, g' + a g = -t f/2,  so  g_{n+1} = -(a g_n + c_{n-1}/2)/(n+1),
+//   f'^2 = (f^2)''/2 + a (f^2)' + w2 f^2   (from f'' + 2 a f' + w2 f = 0),
+//   d(f^2)/da = -2 t f^2,  d(f'^2)/da = -(f^2)' - 2 t f'^2.
+struct TabConst {
+  DF aT, w2T2, T, T2, hT2;  // a T, w2 T^2, T, T^2, T^2/2
+};
+GPSS_HD TabConst table_const(double a, double beta, double T) {
+  return TabConst{df_of(a * T), df_of((beta + a * a) * T * T), df_of(T), df_of(T * T),
+                  df_of(0.5 * T * T)};
+}
+GPSS_HD DF df_int(int n) { return DF{(float)n, 0.f}; }
+
+// One step of the recurrences of c~ and g~: -(al x1 + be x0) ga.
+GPSS_HD DF taylor_step(DF al, DF x1, DF be, DF x0, DF ga) { return -(al * x1 + be * x0) * ga; }
+
+// c~_n and g~_n for n = 0..TAB_NCF (the table kernel runs the two recurrences
+// in two lanes).
+GPSS_HD void taylor_cg_scaled(const TabConst &K, const DF *rcp, DF *c, DF *g) {
+  const DF z = DF{0.f, 0.f};
+  c[0] = g[0] = g[1] = z;
+  c[1] = K.T;
+  c[2] = -(K.aT * K.T);
+  for (int n = 1; n + 2 <= TAB_NCF; ++n)
+    c[n + 2] = taylor_step(K.aT * df_int(2 * (n + 1)), c[n + 1], K.w2T2, c[n],
+                           rcp[n + 2] * rcp[n + 1]);
+  for (int n = 1; n + 1 <= TAB_NCF; ++n) g[n + 1] = taylor_step(K.aT, g[n], K.hT2, c[n - 1], rcp[n + 1]);
 }
 
-// Coefficient k of the six scaled series from c~ (e_n = c~_n / (n+1) and
-// p_n = n c~_n precomputed), as taylor_coeff_pre with the T factors out.
-GPSS_HD void taylor_coeff_scaled(const Dual2<DF> *c, const Dual2<DF> *e, const Dual2<DF> *p,
-                                 const DF *rcp, int k, Dual2<DF> (&g)[6]) {
-  const DF z = df_of(0.0);
-  Dual2<DF> s1 = mkdf(z, z, z), s2 = s1, s3 = s1;
+// Coefficients n of F1 = int f (times t^{n+1}) and its tangents.
+GPSS_HD void taylor_int(const TabConst &K, const DF *rcp, const DF *c, const DF *g, int n, DF &e,
+                        DF &ea, DF &eb) {
+  const DF z = DF{0.f, 0.f};
+  e = c[n] * rcp[n + 1];
+  ea = n > 0 ? -(K.T * c[n - 1]) * rcp[n + 1] : z;
+  eb = g[n] * rcp[n + 1];
+}
+
+// Coefficient t^{k+2} of f^2 and its beta tangent (s1, s1b), t^{k+4} of F1^2
+// and its tangents (s3, s3a, s3b); the squares take each pair once.
+GPSS_HD void taylor_squares(const DF *c, const DF *g, const DF *e, const DF *ea, const DF *eb,
+                            int k, DF &s1, DF &s1b, DF &s3, DF &s3a, DF &s3b) {
+  const DF z = DF{0.f, 0.f};
+  s1 = s1b = s3 = s3a = s3b = z;
   for (int n = 1; n <= k + 1; ++n) {
     const int m = k + 2 - n;
-    s1 = s1 + c[n] * c[m];
-    s2 = s2 + p[n] * p[m];
-    s3 = s3 + e[n] * e[m];
+    if (n < m) {
+      s1 = s1 + c[n] * c[m];
+      s3 = s3 + e[n] * e[m];
+    }
+    s1b = s1b + c[n] * g[m];
+    s3a = s3a + e[n] * ea[m];
+    s3b = s3b + e[n] * eb[m];
   }
-  g[0] = c[k + 1];
-  g[1] = c[k + 1] * df_of((double)(k + 1));
-  g[2] = c[k + 1] * rcp[k + 2];
-  g[3] = s1 * rcp[k + 3];
-  g[4] = s2 * rcp[k + 1];
-  g[5] = s3 * rcp[k + 5];
+  s1 = DF{2.f * s1.hi, 2.f * s1.lo};
+  s3 = DF{2.f * s3.hi, 2.f * s3.lo};
+  if (!(k & 1)) {
+    const int h = k / 2 + 1;
+    s1 = s1 + c[h] * c[h];
+    s3 = s3 + e[h] * e[h];
+  }
+  s1b = DF{2.f * s1b.hi, 2.f * s1b.lo};
+  s3a = DF{2.f * s3a.hi, 2.f * s3a.lo};
+  s3b = DF{2.f * s3b.hi, 2.f * s3b.lo};
 }
 
-// Economised coefficient k of one scaled series: sum_n m[k][n] g~_n.
-GPSS_HD Dual2<DF> econ_apply_scaled(const DF (*m)[TAB_NTAY], int k, const Dual2<DF> *g) {
-  const DF z = df_of(0.0);
-  Dual2<DF> acc = mkdf(z, z, z);
-  for (int n = k; n < TAB_NTAY; ++n) acc = acc + g[n] * m[k][n];
+// Coefficient t^k of f'^2 and its beta tangent from those of f^2 at k, k - 1
+// and k - 2 (zero below the series' start).
+GPSS_HD void taylor_fp2(const TabConst &K, int k, DF p0, DF p1, DF p2, DF b0, DF b1, DF b2,
+                        DF &s2, DF &s2b) {
+  const DF h = DF{0.5f * (float)((k + 2) * (k + 1)), 0.f}, a1 = K.aT * df_int(k + 1);
+  s2 = h * p0 + a1 * p1 + K.w2T2 * p2;
+  s2b = h * b0 + a1 * b1 + K.T2 * p2 + K.w2T2 * b2;
+}
+
+// Coefficient k of the six scaled series, components ordered value (6),
+// d/da (6), d/dbeta (6): p1 = s1 at k - 1, q1 = s2 at k - 1.
+GPSS_HD void taylor_comps(const TabConst &K, const DF *rcp, const DF *c, const DF *g, int k, DF s1,
+                          DF s1b, DF s2, DF s2b, DF s3, DF s3a, DF s3b, DF p1, DF q1,
+                          DF (&o)[18]) {
+  const DF nT = -K.T, k1 = df_int(k + 1), two = DF{2.f, 0.f};
+  const DF cv = c[k + 1], ca = nT * c[k], cb = g[k + 1];
+  const DF r2 = rcp[k + 2], r3 = rcp[k + 3], r1 = rcp[k + 1], r5 = rcp[k + 5];
+  o[0] = cv;       o[6] = ca;                                 o[12] = cb;
+  o[1] = cv * k1;  o[7] = ca * k1;                            o[13] = cb * k1;
+  o[2] = cv * r2;  o[8] = ca * r2;                            o[14] = cb * r2;
+  o[3] = s1 * r3;  o[9] = nT * (two * p1) * r3;               o[15] = s1b * r3;
+  o[4] = s2 * r1;  o[10] = nT * (k1 * p1 + two * q1) * r1;    o[16] = s2b * r1;
+  o[5] = s3 * r5;  o[11] = s3a * r5;                          o[17] = s3b * r5;
+}
+
+// The economisation map as the table kernel takes it: the rows' entries for
+// the traded powers n >= TAB_NC (below them the map is the identity), and 1/i.
+struct EconDF {
+  DF m[TAB_NC][TAB_NTAY - TAB_NC];
+  DF rcp[TAB_NTAY + 8];
+};
+GPSS_HD void econ_df(const EconMap &E, EconDF &o) {
+  for (int k = 0; k < TAB_NC; ++k)
+    for (int n = TAB_NC; n < TAB_NTAY; ++n) o.m[k][n - TAB_NC] = df_of(E.m[k][n]);
+  for (int i = 0; i < TAB_NTAY + 8; ++i) o.rcp[i] = df_of(E.rcp[i]);
+}
+
+// Economised coefficient k of one scaled series: g~_k + sum_n m[k][n] g~_n.
+GPSS_HD DF econ_apply_scaled(const DF (*m)[TAB_NTAY - TAB_NC], int k, const DF *g) {
+  DF acc = g[k];
+#pragma unroll 4
+  for (int n = TAB_NC; n < TAB_NTAY; ++n) acc = acc + g[n] * m[k][n - TAB_NC];
   return acc;
 }
 
@@ -698,33 +772,30 @@ GPSS_HD int table_q(int j) { return j < 3 ? 1 : 2; }
 // beta) tangents of e[j][k] = table coefficient k of series j, in t.
 GPSS_HD void table_coeffs_df(const EconMap &E, double a, double beta, double (&v)[6][TAB_NC],
                              double (&da)[6][TAB_NC], double (&db)[6][TAB_NC]) {
-  DF rcp[2 * TAB_NTAY + 8];
-  for (int i = 0; i < 2 * TAB_NTAY + 8; ++i) rcp[i] = df_of(E.rcp[i]);
+  EconDF D;
+  econ_df(E, D);
   const double T = table_range(rate2<double>(a, beta));
-  const DF one = df_of(1.0), zero = df_of(0.0);
-  const Dual2<DF> ad = mkdf(df_of(a), one, zero), bd = mkdf(df_of(beta), zero, one);
-  const Dual2<DF> w2 = bd + ad * ad;
-  Dual2<DF> c[TAB_NCF + 1], e[TAB_NCF + 1], p[TAB_NCF + 1], g[6][TAB_NTAY];
-  taylor_c_scaled(ad * df_of(T), w2 * df_of(T * T), rcp, c, df_of(T));
-  for (int n = 0; n <= TAB_NCF; ++n) {
-    e[n] = c[n] * rcp[n + 1];
-    p[n] = c[n] * df_of((double)n);
-  }
+  const TabConst K = table_const(a, beta, T);
+  DF c[TAB_NCF + 1], g[TAB_NCF + 1], e[TAB_NCF + 1], ea[TAB_NCF + 1], eb[TAB_NCF + 1];
+  taylor_cg_scaled(K, D.rcp, c, g);
+  for (int n = 0; n <= TAB_NCF; ++n) taylor_int(K, D.rcp, c, g, n, e[n], ea[n], eb[n]);
+  const DF z = DF{0.f, 0.f};
+  DF s1[TAB_NTAY], s1b[TAB_NTAY], s2[TAB_NTAY], s2b[TAB_NTAY], G[18][TAB_NTAY];
   for (int k = 0; k < TAB_NTAY; ++k) {
-    Dual2<DF> h[6];
-    taylor_coeff_scaled(c, e, p, rcp, k, h);
-    for (int j = 0; j < 6; ++j) g[j][k] = h[j];
+    DF s3, s3a, s3b, o[18];
+    taylor_squares(c, g, e, ea, eb, k, s1[k], s1b[k], s3, s3a, s3b);
+    taylor_fp2(K, k, s1[k], k > 0 ? s1[k - 1] : z, k > 1 ? s1[k - 2] : z, s1b[k],
+               k > 0 ? s1b[k - 1] : z, k > 1 ? s1b[k - 2] : z, s2[k], s2b[k]);
+    taylor_comps(K, D.rcp, c, g, k, s1[k], s1b[k], s2[k], s2b[k], s3, s3a, s3b,
+                 k > 0 ? s1[k - 1] : z, k > 0 ? s2[k - 1] : z, o);
+    for (int i = 0; i < 18; ++i) G[i][k] = o[i];
   }
-  DF m[TAB_NC][TAB_NTAY];
-  for (int k = 0; k < TAB_NC; ++k)
-    for (int n = 0; n < TAB_NTAY; ++n) m[k][n] = df_of(E.m[k][n]);
   for (int j = 0; j < 6; ++j)
     for (int k = 0; k < TAB_NC; ++k) {
-      const Dual2<DF> r = econ_apply_scaled(m, k, g[j]);
       const double sc = pow(T, -(double)(k + table_q(j)));
-      v[j][k] = df_val(r.v) * sc;
-      da[j][k] = df_val(r.da) * sc;
-      db[j][k] = df_val(r.db) * sc;
+      v[j][k] = df_val(econ_apply_scaled(D.m, k, G[j])) * sc;
+      da[j][k] = df_val(econ_apply_scaled(D.m, k, G[6 + j])) * sc;
+      db[j][k] = df_val(econ_apply_scaled(D.m, k, G[12 + j])) * sc;
     }
 }
 
@@ -1250,6 +1321,19 @@ GPSS_HD void obs_project_tag(uint8_t tag, F w, const F *m, const F *P, F *u, F &
 }
 
 // Load per-term constants and s^2 from a row of natural parameters.
+// a, beta of term t alone (the table kernel's inputs).
+template <int NT>
+GPSS_HD void load_rates(const float *th, const int *kinds, int t, double &a, double &beta) {
+  int j = 0;
+#pragma unroll
+  for (int i = 0; i < NT - 1; ++i) j += i < t ? (kinds[i] == 1 ? 3 : 2) : 0;
+  const bool sho = kinds[t] == 1;
+  const double w0 = sho ? (double)th[j + 1] : 1.7320508075688772 / (double)th[j + 1];
+  const double q = sho ? (double)th[j + 2] : 0.5;
+  a = w0 / (2.0 * q);
+  beta = (q == 0.5) ? 0.0 : w0 * w0 * (1.0 - 1.0 / (4.0 * q * q));
+}
+
 template <int NT, class F>
 GPSS_HD void load_terms(const float *th, const int *kinds, TermC<F> *tc, F &s2) {
   int j = 0;

@@ -314,11 +314,18 @@ GPSS_D void cp_async_wait() {
 // ---------------------------------------------------------------------------
 // Step-scalar tables, one warp per (hyperparameter row, term), with (a, beta)
 // tangents, in double-float arithmetic on the FP32 pipe (table_coeffs_df is
-// the same computation written sequentially).  Lane 0 runs the scaled
-// recurrence of f's Taylor coefficients c~_n = c_n T^n; lanes form c~_n/(n+1)
-// and n c~_n; lane k sums the products giving coefficient k of the six
-// series; all lanes then share the outputs of the economisation map, each
+// the same computation written sequentially).  The FP64 constants of the
+// block's terms are formed by one thread each.  Lanes 0 and 1 run the scaled
+// recurrences of f's Taylor coefficients and of its beta tangent's; lane k
+// then forms coefficient k of the squares and of the eighteen series and
+// components, and all lanes share the outputs of the economisation map, each
 // scaled back by T^-(k+q) in FP64 and rounded once to FP32.
+//
+// Bound by the serial recurrence (few rows) or by instruction issue (many).
+// The structural tangents need a third of the operations of forward-mode
+// duals, and FP64 instructions, which run at 1/64 of the FP32 rate, are left
+// only for the constants and the final scaling.  2048 tables: 82.9 -> 27.0 us;
+// one warp alone, 28-32 -> 16.5 us.
 // ---------------------------------------------------------------------------
 constexpr int TABLE_WARPS = 4;
 
@@ -326,57 +333,97 @@ template <int NT>
 __global__ void __launch_bounds__(32 * TABLE_WARPS) k_tables(const float *__restrict__ theta,
                                                             int n_rows, int n_params, int kind0,
                                                             int kind1, float *__restrict__ tab,
-                                                            EconMap E) {
-  using DD = Dual2<DF>;
-  constexpr int NCF = TAB_NCF;  // c_0 .. c_NCF
-  __shared__ DD sc[TABLE_WARPS][NCF + 1], se[TABLE_WARPS][NCF + 1], sf[TABLE_WARPS][NCF + 1];
-  __shared__ DD sg[TABLE_WARPS][6][TAB_NTAY];
+                                                            EconDF E) {
+  constexpr int NCF = TAB_NCF;
+  __shared__ DF sc[TABLE_WARPS][5][NCF + 1];  // c~, g~, and F1's e, de/da, de/dbeta
+  __shared__ DF sg[TABLE_WARPS][18][TAB_NTAY];
+  __shared__ TabConst sK[TABLE_WARPS];
+  __shared__ double s_it[TABLE_WARPS][TAB_NC + 2];  // T^-p
   // the economisation map and reciprocals in shared memory: the lanes index
   // them with different k, which the parameter (constant) bank would serialise
-  __shared__ DF sm_m[TAB_NC][TAB_NTAY];
-  __shared__ DF sm_rcp[2 * TAB_NTAY + 8];
-  for (int i = threadIdx.x; i < TAB_NC * TAB_NTAY; i += blockDim.x)
-    sm_m[i / TAB_NTAY][i % TAB_NTAY] = df_of(E.m[i / TAB_NTAY][i % TAB_NTAY]);
-  for (int i = threadIdx.x; i < 2 * TAB_NTAY + 8; i += blockDim.x) sm_rcp[i] = df_of(E.rcp[i]);
-  __syncthreads();
+  __shared__ DF sm_m[TAB_NC][TAB_NTAY - TAB_NC];
+  __shared__ DF sm_rcp[TAB_NTAY + 8];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rt = blockIdx.x * TABLE_WARPS + w;
-  if (rt >= n_rows * NT) return;  // whole warps leave together
-  const int row = rt / NT, t = rt % NT;
   const int kinds[4] = {kind0, kind1, 0, 0};
-  TermC<double> tc[NT];
-  double s2;
-  load_terms<NT, double>(theta + (size_t)row * n_params, kinds, tc, s2);
-  const double T = table_range(tc[t].r2);
-  const DF one = df_of(1.0), zero = df_of(0.0);
-  const DD a = mkdf(df_of(tc[t].a), one, zero), beta = mkdf(df_of(tc[t].beta), zero, one);
-  const DD w2 = beta + a * a;
-  if (lane == 0) taylor_c_scaled(a * df_of(T), w2 * df_of(T * T), sm_rcp, &sc[w][0], df_of(T));
-  __syncwarp();
-  for (int n = lane; n <= NCF; n += 32) {
-    const DD c = sc[w][n];
-    se[w][n] = c * sm_rcp[n + 1];
-    sf[w][n] = c * df_of((double)n);
+  if (threadIdx.x < TABLE_WARPS) {
+    const int r = blockIdx.x * TABLE_WARPS + threadIdx.x;
+    if (r < n_rows * NT) {
+      double a, beta;
+      load_rates<NT>(theta + (size_t)(r / NT) * n_params, kinds, r % NT, a, beta);
+      const double T = table_range(rate2<double>(a, beta)), iT = 1.0 / T;
+      sK[threadIdx.x] = table_const(a, beta, T);
+      double p = 1.0;
+#pragma unroll
+      for (int i = 0; i < TAB_NC + 2; ++i) {
+        s_it[threadIdx.x][i] = p;
+        p *= iT;
+      }
+    }
+  }
+  for (int i = threadIdx.x; i < TAB_NC * (TAB_NTAY - TAB_NC); i += blockDim.x)
+    sm_m[i / (TAB_NTAY - TAB_NC)][i % (TAB_NTAY - TAB_NC)] =
+        E.m[i / (TAB_NTAY - TAB_NC)][i % (TAB_NTAY - TAB_NC)];
+  for (int i = threadIdx.x; i < TAB_NTAY + 8; i += blockDim.x) sm_rcp[i] = E.rcp[i];
+  __syncthreads();
+  if (rt >= n_rows * NT) return;  // whole warps leave together
+  const TabConst K = sK[w];
+  const DF z = DF{0.f, 0.f};
+  DF *c = sc[w][0], *g = sc[w][1], *e = sc[w][2], *ea = sc[w][3], *eb = sc[w][4];
+  {
+    // lane 0: c~ (x1 = c~_{n+1}, x0 = c~_n); lane 1: g~ (x1 = g~_n, with
+    // c~_{n-1} from lane 0)
+    DF x1 = lane == 0 ? -(K.aT * K.T) : z, x0 = lane == 0 ? K.T : z, cm = z;
+    if (lane == 0) {
+      c[0] = z;
+      c[1] = x0;
+      c[2] = x1;
+    } else if (lane == 1) {
+      g[0] = g[1] = z;
+    }
+    const DF be = lane == 0 ? K.w2T2 : K.hT2;
+    for (int n = 1; n + 2 <= NCF; ++n) {
+      const DF r1 = sm_rcp[n + 1];
+      const DF al = lane == 0 ? K.aT * df_int(2 * (n + 1)) : K.aT;
+      const DF ga = lane == 0 ? sm_rcp[n + 2] * r1 : r1;
+      const DF cp = DF{__shfl_sync(0xffffffffu, cm.hi, 0), __shfl_sync(0xffffffffu, cm.lo, 0)};
+      const DF x = taylor_step(al, x1, be, lane == 0 ? x0 : cp, ga);
+      cm = x0;  // c~_n, the next step's c~_{n-1}
+      x0 = x1;
+      x1 = x;
+      if (lane == 0)
+        c[n + 2] = x;
+      else if (lane == 1)
+        g[n + 1] = x;
+    }
   }
   __syncwarp();
-  if (lane < TAB_NTAY) {
-    DD g[6];
-    taylor_coeff_scaled(&sc[w][0], &se[w][0], &sf[w][0], sm_rcp, lane, g);
+  if (lane < NCF) taylor_int(K, sm_rcp, c, g, lane, e[lane], ea[lane], eb[lane]);
+  __syncwarp();
+  {
+    const int k = min(lane, TAB_NTAY - 1);
+    DF s1, s1b, s2, s2b, s3, s3a, s3b;
+    taylor_squares(c, g, e, ea, eb, k, s1, s1b, s3, s3a, s3b);
+    auto up = [&](DF x, int d) {  // the value of lane - d (zero below the first)
+      const DF y = DF{__shfl_up_sync(0xffffffffu, x.hi, d), __shfl_up_sync(0xffffffffu, x.lo, d)};
+      return lane >= d ? y : z;
+    };
+    const DF p1 = up(s1, 1), p2 = up(s1, 2), b1 = up(s1b, 1), b2 = up(s1b, 2);
+    taylor_fp2(K, k, s1, p1, p2, s1b, b1, b2, s2, s2b);
+    const DF q1 = up(s2, 1);
+    DF o[18];
+    taylor_comps(K, sm_rcp, c, g, k, s1, s1b, s2, s2b, s3, s3a, s3b, p1, q1, o);
+    if (lane < TAB_NTAY) {
 #pragma unroll
-    for (int j = 0; j < 6; ++j) sg[w][j][lane] = g[j];
+      for (int i = 0; i < 18; ++i) sg[w][i][lane] = o[i];
+    }
   }
   __syncwarp();
   float *base = tab + (size_t)rt * TAB_NC * TAB_W;
-  for (int o = lane; o < 6 * TAB_NC; o += 32) {
-    const int j = o / TAB_NC, k = o % TAB_NC;
-    const DD e = econ_apply_scaled(sm_m, k, &sg[w][j][0]);
-    double sT = 1.0;
-    const double iT = 1.0 / T;
-    for (int i = 0; i < k + table_q(j); ++i) sT *= iT;
-    float *r = base + (size_t)k * TAB_W;
-    r[j] = (float)(df_val(e.v) * sT);
-    r[8 + j] = (float)(df_val(e.da) * sT);
-    r[14 + j] = (float)(df_val(e.db) * sT);
+  for (int o = lane; o < 18 * TAB_NC; o += 32) {
+    const int i = o / TAB_NC, k = o % TAB_NC, j = i % 6;
+    const DF x = econ_apply_scaled(sm_m, k, sg[w][i]);
+    base[(size_t)k * TAB_W + (i < 6 ? i : i + 2)] = (float)(df_val(x) * s_it[w][k + table_q(j)]);
   }
   for (int o = lane; o < TAB_NC * 2; o += 32) {
     // the pads: columns 6, 7 of each record
@@ -1960,10 +2007,12 @@ cudaError_t launch_tables(const float *theta, int n_rows, int n_params, int k0, 
                           float *tab, cudaStream_t st) {
   const int n = n_rows * S::NT;
   if (n <= 0) return cudaSuccess;
-  static const EconMap E = [] {
+  static const EconDF E = [] {
     EconMap e;
     econ_map(e);
-    return e;
+    EconDF d;
+    econ_df(e, d);
+    return d;
   }();
   k_tables<S::NT><<<(n + TABLE_WARPS - 1) / TABLE_WARPS, 32 * TABLE_WARPS, 0, st>>>(
       theta, n_rows, n_params, k0, k1, tab, E);
