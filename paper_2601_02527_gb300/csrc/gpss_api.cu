@@ -41,7 +41,7 @@ CombineOps comb64_2_3_0();
 __global__ void k_series_sum(int n_out, int per_series, int n_series, int n_chunks,
                              const int32_t *__restrict__ ch_first,
                              const double *__restrict__ ll_part, int n_vch,
-                             const float *__restrict__ gpart, int n_params,
+                             const float *__restrict__ gpart, int n_seg, int n_params,
                              double *__restrict__ ll_out, float *__restrict__ grad_out) {
   // one warp per output row; lanes stride over the row's chunks and a fixed
   // shuffle tree combines them (the same order on every call)
@@ -60,8 +60,10 @@ __global__ void k_series_sum(int n_out, int per_series, int n_series, int n_chun
   if (gpart) {
     for (int p = 0; p < n_params; ++p) {
       double acc = 0.0;
-      const float *g = gpart + (size_t)p * n_vch + base;
-      for (int c = c0 + lane; c < c1; c += 32) acc += (double)g[c];
+      for (int q = 0; q < n_seg; ++q) {
+        const float *g = gpart + ((size_t)q * n_params + p) * n_vch + base;
+        for (int c = c0 + lane; c < c1; c += 32) acc += (double)g[c];
+      }
       for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
       if (lane == 0) grad_out[(size_t)v * n_params + p] = (float)acc;
     }
@@ -237,6 +239,7 @@ struct GraphKey {
 
 struct gp_ss_model {
   int device = 0;
+  int n_sm = 0;  // multiprocessors of the device
   int n_series = 0, n_terms = 0, kinds[4] = {0, 0, 0, 0}, layout = 0, n_slots = 1;
   bool product = false;  // a product term (instantaneous measurements only)
   bool mixed = false;    // instantaneous measurements among exposure averages
@@ -894,6 +897,33 @@ struct ElemSlices {
   const cudaEvent_t *ready;
 };
 
+// Segments of ck events per chunk that the gradient walks in parallel, one
+// thread each (1: one thread per chunk walks them in turn).  A thread takes
+// the serial time of its events, so too few chunks leave the GPU idle;
+// parallel segments cost each segment's own element beside the chunk's and a
+// boundary adjoint per segment.  The line lies where both take the same time:
+// 6 warps of chunks per SM, 12 for states of at most 4 (cheaper elements).
+// One call, parallel against in turn, 152 SMs: two SHO terms 911 warps 1254
+// us against 1367, 1215 warps 1534 against 1418; SHO + Matern-3/2 with three
+// slots 624 warps 1674 against 1935, 936 warps 2136 each; instants 1205
+// warps 1009 against 1152, 1649 warps 1279 against 1300.  The adjoint at a
+// segment's end differs from the walked one in rounding; exposure gradients
+// and predictions, differences of nearly equal terms, would show it at 3e-5
+// of their size and keep the walk in turn.
+int grad_segments(const gp_ss_model *m, int n_vch, int ck) {
+  constexpr int kMaxSegments = 1024;  // k_seg_info carries the adjoints back through them in turn
+  constexpr size_t kMaxReplay = (size_t)2 << 30;  // bytes of the replay buffers
+  // shorter segments would put a boundary adjoint's rounding every few events
+  if (m->product || ck < 32) return 1;
+  const OpTable &o = m->ops;
+  const int n_seg = (m->max_chunk + ck - 1) / ck;
+  const int per_sm = o.D <= 4 ? 12 : 6;
+  if (n_vch / 32 > per_sm * m->n_sm || n_seg < 2 || n_seg > kMaxSegments) return 1;
+  const size_t replay =
+      (size_t)n_seg * ck * (4 * ((o.D + o.NP + 3) / 4)) * n_vch * sizeof(float);
+  return replay <= kMaxReplay ? n_seg : 1;
+}
+
 // Enqueue the log-likelihood (and optionally gradient) computation.
 gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int per_series,
                      double *ll, float *grad, cudaStream_t st, float *dexp = nullptr,
@@ -962,6 +992,8 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
     return true;
   };
   float *ef = nullptr, *adj = nullptr, *ckpt = nullptr, *gpart = nullptr, *tabs = nullptr;
+  float *segel = nullptr, *seg_info = nullptr, *seg_adj = nullptr, *rbuf = nullptr;
+  int n_gpart = 1;
   void *state_end = nullptr, *info = nullptr, *scratch = nullptr;
   double *ed = nullptr, *ll_part = nullptr;
   gp_ss_status res = GP_SS_OK;
@@ -970,6 +1002,8 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
     // every recomputation segment but a chunk's first
     const int ck = m->ckpt_interval;
     const int n_pck = std::max((m->max_chunk - 1) / ck, 1);
+    int n_seg = grad && tree && !dexp && !pred ? grad_segments(m, n_vch, ck) : 1;
+    const size_t replay = (size_t)ck * (4 * ((SD + 3) / 4)) * n_vch * sizeof(float);
     if (!grab((void **)&ef, (size_t)o.NF * n_vch * sizeof(float)) ||
         !grab((void **)&ed, (size_t)o.ND * n_vch * sizeof(double)) ||
         !grab((void **)&tabs, (size_t)n_sets * o.NT * gpss::TAB_TERM * sizeof(float)) ||
@@ -989,6 +1023,20 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
         break;
       }
     }
+    if (n_seg > 1) {
+      // without the memory for parallel segments they are walked in turn
+      const size_t before = bufs.size(), rec = (size_t)(n_seg - 1) * n_vch * sizeof(float);
+      if (!grab((void **)&segel, rec * o.NF) || !grab((void **)&seg_info, rec * SD) ||
+          !grab((void **)&seg_adj, rec * SD) || !grab((void **)&rbuf, replay * n_seg)) {
+        while (bufs.size() > before) {
+          cudaFreeAsync(bufs.back(), st);
+          bufs.pop_back();
+        }
+        cudaGetLastError();
+        segel = seg_info = seg_adj = rbuf = nullptr;
+        n_seg = 1;
+      }
+    }
     {
       PhaseTimer pt(m, st, 0);
       if (o.tables(theta, n_sets, m->n_params, m->kinds[0], m->kinds[1], tabs, st)) {
@@ -1005,7 +1053,7 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
         // on the compute stream, while the copy stream sends the next group
         if (!res && slices && interleave_events(m, c0, cn, st) != cudaSuccess) res = GP_SS_ECUDA;
         if (!res && o.elem(dm, theta, n_vch, per_series, ef, ed, m->d_err, tabs,
-                           grad ? ckpt : nullptr, ck, dcache, c0, cn, st))
+                           grad ? ckpt : nullptr, ck, dcache, c0, cn, segel, n_seg, st))
           res = GP_SS_ECUDA;
       }
       if (res) break;
@@ -1053,7 +1101,7 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
       }
     }
     if (grad) {
-      float *rbuf = nullptr, *gdt = nullptr, *gwe = nullptr;
+      float *gdt = nullptr, *gwe = nullptr;
       float2 *cond = nullptr;
       const int exp_rows = per_series ? 1 : n_sets;
       if ((dexp && (!grab((void **)&gdt, (size_t)exp_rows * m->n_events * sizeof(float)) ||
@@ -1062,9 +1110,8 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
         res = GP_SS_ENOMEM;
         break;
       }
-      if ((!m->product &&
-           !grab((void **)&rbuf, (size_t)ck * (4 * ((SD + 3) / 4)) * n_vch * sizeof(float))) ||
-          !grab((void **)&gpart, (size_t)m->n_params * n_vch * sizeof(float))) {
+      if ((!m->product && !rbuf && !grab((void **)&rbuf, replay)) ||
+          !grab((void **)&gpart, (size_t)n_seg * m->n_params * n_vch * sizeof(float))) {
         res = GP_SS_ENOMEM;
         break;
       }
@@ -1077,8 +1124,12 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
         if (res) break;
       } else {
         const gpss::PredPlan none;
-        if (o.grad(dm, theta, n_vch, per_series, state_end, eb == 8 ? 1 : 0, adj, ckpt, gpart,
-                   m->d_err, tabs, rbuf, dcache, ck, gdt, gwe, cond, pred ? *pred : none, st)) {
+        n_gpart = n_seg;
+        if ((n_seg > 1 && o.seg_adjoint(dm, n_vch, state_end, info, eb == 8 ? 1 : 0, ckpt, segel,
+                                        seg_info, seg_adj, ck, n_seg, st)) ||
+            o.grad(dm, theta, n_vch, per_series, state_end, eb == 8 ? 1 : 0, adj, ckpt, gpart,
+                   m->d_err, tabs, rbuf, dcache, ck, gdt, gwe, cond, pred ? *pred : none,
+                   seg_adj, n_seg, st)) {
           res = GP_SS_ECUDA;
           break;
         }
@@ -1110,7 +1161,7 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
       PhaseTimer pt(m, st, 3);
       gpss::k_series_sum<<<(n_out * 32 + 127) / 128, 128, 0, st>>>(
           n_out, per_series, m->n_series, m->n_chunks, m->d_ch_first, tree ? ll_part : nullptr,
-          n_vch, grad ? gpart : nullptr, m->n_params, ll, grad);
+          n_vch, grad ? gpart : nullptr, n_gpart, m->n_params, ll, grad);
       GPSS_COUNT_LAUNCH();
       if (cudaGetLastError() != cudaSuccess) res = GP_SS_ECUDA;
     }
@@ -1220,6 +1271,7 @@ gp_ss_status gp_ss_build_model(const gp_ss_kernel_spec *spec, int n_series,
   gp_ss_model *m = new (std::nothrow) gp_ss_model();
   if (!m) return GP_SS_ENOMEM;
   cudaGetDevice(&m->device);
+  cudaDeviceGetAttribute(&m->n_sm, cudaDevAttrMultiProcessorCount, m->device);
   m->n_series = n_series;
   m->n_terms = spec->n_terms;
   m->layout = spec->n_terms == 1 ? 0 : spec->integral_layout;
@@ -1621,10 +1673,8 @@ gp_ss_status gp_ss_loglik_grad_host(const gp_ss_model *m, const float *theta_hos
   // 1.84 ms with four, 1.90 ms with two; 11424 chunks: the whole call 1.75 ms
   // with four, 1.17 ms with one).
   constexpr int kGroups = 4;
-  int n_sm = 0;
-  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, m->device);
   const int n_groups =
-      std::max(1, std::min(kGroups, m->n_chunks / std::max(1, n_sm * gpss::ELEM_BS)));
+      std::max(1, std::min(kGroups, m->n_chunks / std::max(1, m->n_sm * gpss::ELEM_BS)));
   cudaStream_t cs = nullptr;
   cudaEvent_t start_ev = nullptr, ready[kGroups] = {};
   int c0[kGroups + 1] = {};
@@ -1735,7 +1785,7 @@ gp_ss_status gp_ss_span_element(const gp_ss_model *m, const float *theta, int n_
     res = GP_SS_ENOMEM;
   } else if (o.tables(theta, n_sets, m->n_params, m->kinds[0], m->kinds[1], tabs, st) ||
              o.elem(dm, theta, n_vch, theta_per_series, ef, ed, m->d_err, tabs, nullptr, 0,
-                    nullptr, c_begin, c_end - c_begin, st) ||
+                    nullptr, c_begin, c_end - c_begin, nullptr, 0, st) ||
              o.span_element(ef, ed, n_vch, m->n_chunks, c_begin, c_end, rows, scratch, elem_out,
                             st)) {
     res = GP_SS_ECUDA;
@@ -2074,7 +2124,7 @@ extern "C" gp_ss_status gp_ss_loglik_noalloc(const gp_ss_model *m, const float *
   // so nothing in the shared array needs clearing between calls
   if (o.tables(theta, n_sets, m->n_params, m->kinds[0], m->kinds[1], tabs, st) != cudaSuccess ||
       o.elem(dm, theta, n_vch, theta_per_series, ef, ed, nullptr, tabs, nullptr, 0, nullptr, 0,
-             m->n_chunks, st) !=
+             m->n_chunks, nullptr, 0, st) !=
           cudaSuccess)
     return GP_SS_ECUDA;
   const gpss::CombineOps &cb = m->comb_prec == 64 ? o.comb64 : o.comb32;

@@ -24,7 +24,8 @@
 //                 log-likelihood in closed form, and for the gradient the
 //                 information about each chunk's end state from all later
 //                 data, turned into the adjoint of that state.
-//      k_grad     one thread per chunk, segments of ck events from last to
+//      k_grad     one thread per chunk (or per segment, where chunks are too
+//                 few to fill the GPU), segments of ck events from last to
 //                 first: the segment's starting state from the partial
 //                 element k_elem saved there and the chunk's incoming state,
 //                 a forward replay of the segment, then a sweep back in time
@@ -617,7 +618,7 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
                                               const float *__restrict__ tabs,
                                               float *__restrict__ pck, int ck,
                                               float *__restrict__ dcache, int c_begin,
-                                              int c_count) {
+                                              int c_count, float *__restrict__ segel) {
   using F = float;
   constexpr int D = S::D;
   using L = ElemLayout<S>;
@@ -639,9 +640,16 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
   // OD = true launch, the others in the OD = false one (whole warps: a warp's
   // chunks share one row)
   if ((any_overdamped<S::NT>(tc) || M.mixed) != OD) return;
+  // blocks y > 0: the element of the chunk's segment y - 1 alone (counted from
+  // the chunk's end), for the gradient with one thread per segment
+  const int seg = (int)blockIdx.y - 1;
+  const int len = M.ch_len[c];
+  const int k_hi = seg < 0 ? len : len - seg * ck;
+  const int k_lo = seg < 0 ? 0 : k_hi - ck;
   const float4 *tab =
       stage_table<S::NT>(tabs, row, smem_tab + (threadIdx.x >> 5) * (S::NT * TAB_TERM / 4));
-  const bool first = M.ch_flags[c] & 1;
+  if (seg >= 0 && k_lo <= 0) return;  // nothing precedes the first segment
+  const bool first = seg < 0 && (M.ch_flags[c] & 1);
   F A[D][D], b[D], C[S::NP], eta[D], J[S::NP];
   if (first) {
     init_state<S>(tc, b, C);
@@ -662,15 +670,14 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
   double gam = 0.0, ld = 0.0;
   int n_end = 0;
   bool bad = false;
-  const int len = M.ch_len[c];
-  float4 *dc = dcache_col<S::NT>(M, dcache, vc);
+  float4 *dc = dcache_col<S::NT>(M, seg < 0 ? dcache : nullptr, vc);
   EventReader rd;
-  rd.start(M, c, 0, len);
+  rd.start(M, c, k_lo, k_hi);
   // gradient segments end at len - j ck (the first one is the short one);
   // at each later segment's start the partial element is saved
   const int f0 = len - ((len - 1) / ck) * ck;
-  int next_ck = pck ? f0 : len;
-  for (int kk = 0; kk < len; ++kk) {
+  int next_ck = pck && seg < 0 ? f0 : len;
+  for (int kk = k_lo; kk < k_hi; ++kk) {
     if (kk == next_ck) {
       float *dst = pck + (size_t)((kk - f0) / ck) * (L::NF + 1) * n_vch;
       store_elem<S>(dst, n_vch, vc, A, b, C, eta, J);
@@ -706,6 +713,11 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
       }
     }
     elem_event<S, F, OD>(B, tag, q.x, q.y, q.z, s2, A, b, C, eta, J, gam, ld, n_end, bad);
+  }
+  if (seg >= 0) {
+    store_elem<S>(segel + (size_t)seg * L::NF * n_vch, n_vch, vc, A, b, C, eta, J);
+    if (bad) flag_error(err, orow, 7);
+    return;
   }
   store_elem<S>(ef, n_vch, vc, A, b, C, eta, J);
   ed[vc] = gam;
@@ -1394,13 +1406,80 @@ GPSS_HD void apply_partial(const float *src, int n_vch, int vc, const float *m_i
   }
 }
 
+// Gradient with one thread per segment: the adjoint of the filtered state at
+// the end of every segment but a chunk's last, by the same identities as at
+// chunk boundaries.
+// k_seg_info, one thread per chunk: the information about the state at a
+// segment's end from all later data, carried back through the later
+// segments' own elements segel (record q: the segment q from the chunk's
+// end); seg_info record q: the end of segment q + 1.  k_seg_adjoint, one
+// thread per segment: the state there from the partial element, then the
+// adjoint, record q - 1 for segment q.
+template <class S>
+__global__ void __launch_bounds__(64) k_seg_info(DevModel M, int n_vch,
+                                                 const void *__restrict__ info_incl, int se64,
+                                                 const float *__restrict__ segel,
+                                                 float *__restrict__ seg_info, int ck) {
+  using L = ElemLayout<S>;
+  constexpr int D = S::D, SD = D + S::NP;
+  const int vc = blockIdx.x * blockDim.x + threadIdx.x;
+  if (vc >= n_vch) return;
+  const int c = vc % M.n_chunks;
+  const int len = M.ch_len[c];
+  float ie[D], iJ[S::NP];
+  if (M.ch_flags[c] & 2) {
+#pragma unroll
+    for (int i = 0; i < D; ++i) ie[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < S::NP; ++i) iJ[i] = 0.f;
+  } else {
+    load_state_f<S>(info_incl, se64, n_vch, vc + 1, ie, iJ);
+  }
+  for (int q = 0; len - (q + 1) * ck > 0; ++q) {
+    float A[D][D], b[D], C[S::NP], eta[D], J[S::NP];
+    load_elem<S>(segel + (size_t)q * L::NF * n_vch, n_vch, vc, A, b, C, eta, J);
+    info_through<S, float>(A, b, C, eta, J, ie, iJ);
+    store_rec<S>(seg_info + (size_t)q * SD * n_vch, n_vch, vc, ie, iJ);
+  }
+}
+
+template <class S>
+__global__ void __launch_bounds__(64) k_seg_adjoint(DevModel M, int n_vch,
+                                                    const void *__restrict__ state_end, int se64,
+                                                    const float *__restrict__ pck,
+                                                    const float *__restrict__ seg_info,
+                                                    float *__restrict__ seg_adj, int ck) {
+  constexpr int D = S::D, SD = D + S::NP, NF = ElemLayout<S>::NF;
+  const int vc = blockIdx.x * blockDim.x + threadIdx.x;
+  if (vc >= n_vch) return;
+  const int c = vc % M.n_chunks;
+  const int nseg = (M.ch_len[c] + ck - 1) / ck;
+  const int q = blockIdx.y + 1;
+  if (q >= nseg) return;
+  float m[D], P[S::NP], mi[D], Pi[S::NP], ie[D], iJ[S::NP], lam[D], Lam[S::NP];
+  if (M.ch_flags[c] & 1) {
+    // the first chunk's partial elements start from the prior (A = 0)
+#pragma unroll
+    for (int i = 0; i < D; ++i) mi[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < S::NP; ++i) Pi[i] = 0.f;
+  } else {
+    load_state_f<S>(state_end, se64, n_vch, vc - 1, mi, Pi);
+  }
+  apply_partial<S>(pck + (size_t)(nseg - 1 - q) * (NF + 1) * n_vch, n_vch, vc, mi, Pi, m, P);
+  load_rec<S>(seg_info + (size_t)(q - 1) * SD * n_vch, n_vch, vc, ie, iJ);
+  boundary_adjoint<S, float>(m, P, ie, iJ, lam, Lam);
+  store_rec<S>(seg_adj + (size_t)(q - 1) * SD * n_vch, n_vch, vc, lam, Lam);
+}
+
 // Segments of ck events aligned to the chunk's end (the first may be
 // shorter).  Walking the segments from last to first: the filtered state at
 // the segment's start comes from the partial element saved there by k_elem,
 // the segment is replayed forward into this thread's column of rbuf (global,
 // coalesced across the warp; slot k holds (m, P) before the segment's k-th
-// event), then walked backwards in time.  With gdt set, the walk also
-// writes, per event k of theta set r, gdt[r n_events + k] = d loglik / d
+// event), then walked backwards in time.  With seg_adj set (the adjoints at
+// segment ends, k_seg_adjoint), blockIdx.y picks the thread's only segment,
+// counted from the chunk's end.  With gdt set, the walk also writes, per event k of theta set r, gdt[r n_events + k] = d loglik / d
 // (gap before k) and, at an end event, gwe[...] = w^2 d loglik / d w
 // (w = 1/delta of its measurement; dw/dt_start = w^2 = -dw/dt_end).
 template <class S>
@@ -1413,7 +1492,8 @@ __global__ void __launch_bounds__(GRAD_BS, GRAD_MIN_BLOCKS) k_grad(DevModel M, c
                                              float *__restrict__ rbuf,
                                              const float *__restrict__ dcache, int ck,
                                              float *__restrict__ gdt, float *__restrict__ gwe,
-                                             float2 *__restrict__ cond, PredPlan pp) {
+                                             float2 *__restrict__ cond, PredPlan pp,
+                                             const float *__restrict__ seg_adj) {
   using F = float;
   constexpr int D = S::D;
   constexpr int SD = D + S::NP;
@@ -1424,6 +1504,10 @@ __global__ void __launch_bounds__(GRAD_BS, GRAD_MIN_BLOCKS) k_grad(DevModel M, c
   extern __shared__ float sm[];
   const int vc = blockIdx.x * blockDim.x + threadIdx.x;
   if (vc >= n_vch) return;
+  // with seg_adj, this thread's only segment, counted from the chunk's end
+  const int sq = blockIdx.y;
+  rbuf += (size_t)sq * ck * (4 * SG) * n_vch;
+  gpart += (size_t)sq * M.n_params * n_vch;
   const int c = vc % M.n_chunks;
   const int set = vc / M.n_chunks;
   const int s = M.ch_series[c];
@@ -1449,8 +1533,15 @@ __global__ void __launch_bounds__(GRAD_BS, GRAD_MIN_BLOCKS) k_grad(DevModel M, c
     const int len = M.ch_len[c];
     const int nseg = (len + ck - 1) / ck;
     const int f0 = len - (nseg - 1) * ck;
+    if (sq > 0 && sq >= nseg) {  // a shorter chunk: no such segment
+      for (int p = 0; p < M.n_params; ++p) gpart[(size_t)p * n_vch + vc] = 0.f;
+      return;
+    }
+    const int seg_hi = nseg - 1 - sq, seg_lo = seg_adj ? max(seg_hi, 0) : 0;
     F lam[D], Lam[S::NP];
-    if (last) {
+    if (sq > 0) {
+      load_rec<S>(seg_adj + (size_t)(sq - 1) * SD * n_vch, n_vch, vc, lam, Lam);
+    } else if (last) {
   #pragma unroll
       for (int i = 0; i < D; ++i) lam[i] = F(0);
   #pragma unroll
@@ -1468,7 +1559,7 @@ __global__ void __launch_bounds__(GRAD_BS, GRAD_MIN_BLOCKS) k_grad(DevModel M, c
     const size_t rs = (size_t)n_vch;
     const float4 *dc = dcache_col<S::NT>(M, const_cast<float *>(dcache), vc);
     bool bad = false;
-    for (int seg = nseg - 1; seg >= 0; --seg) {
+    for (int seg = seg_hi; seg >= seg_lo; --seg) {
       const int k0 = seg == 0 ? 0 : f0 + (seg - 1) * ck;
       const int k1 = seg == 0 ? f0 : k0 + ck;
       if (seg == 0) {
@@ -1672,7 +1763,7 @@ __global__ void __launch_bounds__(GRAD_BS, GRAD_MIN_BLOCKS) k_grad(DevModel M, c
         }
       }
     }
-    if (first) {
+    if (first && seg_lo == 0) {
       // P0 = blkdiag(var diag(1, w2), I)
   #pragma unroll
       for (int t = 0; t < S::NT; ++t) {
@@ -1725,11 +1816,12 @@ __global__ void __launch_bounds__(GRAD_BS, GRAD_MIN_BLOCKS) k_grad(DevModel M, c
 }
 
 // Ordered per-series sums over chunks (deterministic): log-likelihood parts
-// and gradient parts (field-major, stride n_vch), FP64 accumulation.
+// and gradient parts (n_seg records, field-major, stride n_vch), FP64
+// accumulation.
 __global__ void k_series_sum(int n_out, int per_series, int n_series, int n_chunks,
                              const int32_t *__restrict__ ch_first,
                              const double *__restrict__ ll_part, int n_vch,
-                             const float *__restrict__ gpart, int n_params,
+                             const float *__restrict__ gpart, int n_seg, int n_params,
                              double *__restrict__ ll_out, float *__restrict__ grad_out);
 
 // Exposure-window gradient per measurement (input order) from the per-event
@@ -1945,11 +2037,17 @@ struct OpTable {
   cudaError_t (*plain32)(const DevModel &, const float *, int, int, double *, int *, cudaStream_t);
   cudaError_t (*plain64)(const DevModel &, const float *, int, int, double *, int *, cudaStream_t);
   cudaError_t (*elem)(const DevModel &, const float *, int, int, float *, double *, int *,
-                      const float *, float *, int, float *, int, int, cudaStream_t);
+                      const float *, float *, int, float *, int, int, float *, int,
+                      cudaStream_t);
+  // gradient with one thread per segment: the adjoints at the segments' ends
+  // (null for product models)
+  cudaError_t (*seg_adjoint)(const DevModel &, int, const void *, const void *, int,
+                             const float *, const float *, float *, float *, int, int,
+                             cudaStream_t);
   cudaError_t (*grad)(const DevModel &, const float *, int, int, const void *, int,
                       const float *, const float *, float *, int *, const float *, float *,
                       const float *, int, float *, float *, float2 *, const PredPlan &,
-                      cudaStream_t);
+                      const float *, int, cudaStream_t);
   cudaError_t (*tables)(const float *, int, int, int, int, float *, cudaStream_t);
   CombineOps comb32, comb64;  // the combination in FP32 / FP64
   int NT;
@@ -1983,7 +2081,8 @@ cudaError_t launch_plain(const DevModel &M, const float *theta, int n_out, int p
 template <class S>
 cudaError_t launch_elem(const DevModel &M, const float *theta, int n_vch, int per_series,
                         float *ef, double *ed, int *err, const float *tabs, float *pck, int ck,
-                        float *dcache, int c_begin, int c_count, cudaStream_t st) {
+                        float *dcache, int c_begin, int c_count, float *segel, int n_seg,
+                        cudaStream_t st) {
   if (n_vch <= 0 || c_count <= 0) return cudaSuccess;
   if (c_begin < 0 || c_begin + c_count > M.n_chunks) return cudaErrorInvalidValue;
   if (pck && (ck < 2 || ck > 64 || (ck & 1))) return cudaErrorInvalidValue;
@@ -1992,12 +2091,13 @@ cudaError_t launch_elem(const DevModel &M, const float *theta, int n_vch, int pe
   // two launches: rows without an overdamped term (the lean body), then rows
   // with one; each skips the other's rows
   const int64_t nt = (int64_t)(n_vch / M.n_chunks) * c_count;
-  const int nb = (int)((nt + bs - 1) / bs);
+  // every segment's own element but the first one's beside the chunks'
+  const dim3 nb((unsigned)((nt + bs - 1) / bs), segel ? n_seg : 1);
   k_elem<S, false><<<nb, bs, smem, st>>>(M, theta, n_vch, per_series, ef, ed, err, tabs, pck,
-                                         pck ? ck : 1, dcache, c_begin, c_count);
+                                         pck ? ck : 1, dcache, c_begin, c_count, segel);
   GPSS_COUNT_LAUNCH();
   k_elem<S, true><<<nb, bs, smem, st>>>(M, theta, n_vch, per_series, ef, ed, err, tabs, pck,
-                                        pck ? ck : 1, dcache, c_begin, c_count);
+                                        pck ? ck : 1, dcache, c_begin, c_count, segel);
   GPSS_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -2125,15 +2225,32 @@ cudaError_t launch_grad(const DevModel &M, const float *theta, int n_vch, int pe
                         const void *state_end, int se64, const float *adj_end, const float *pck,
                         float *gpart, int *err, const float *tabs, float *rbuf,
                         const float *dcache, int ck, float *gdt, float *gwe, float2 *cond,
-                        const PredPlan &pp, cudaStream_t st) {
+                        const PredPlan &pp, const float *seg_adj, int n_seg, cudaStream_t st) {
   if (n_vch <= 0) return cudaSuccess;
   if (ck < 2 || ck > 64 || (ck & 1)) return cudaErrorInvalidValue;
   const int SG = (S::D + S::NP + 3) / 4, NDG = DcW<S::NT>::G;
   const size_t smem = (size_t)(GRAD_BS / 32) * S::NT * TAB_TERM * sizeof(float) +
                       (size_t)GRAD_STAGES * (SG + NDG) * GRAD_BS * sizeof(float4);
-  k_grad<S><<<(n_vch + GRAD_BS - 1) / GRAD_BS, GRAD_BS, smem, st>>>(
+  k_grad<S><<<dim3((n_vch + GRAD_BS - 1) / GRAD_BS, seg_adj ? n_seg : 1), GRAD_BS, smem, st>>>(
       M, theta, n_vch, per_series, state_end, se64, adj_end, pck, gpart, err, tabs, rbuf, dcache,
-      ck, gdt, gwe, cond, pp);
+      ck, gdt, gwe, cond, pp, seg_adj);
+  GPSS_COUNT_LAUNCH();
+  return cudaGetLastError();
+}
+
+// Adjoints at segment ends, seg_adj [(n_seg - 1) SD n_vch]; seg_info is
+// scratch of the same size.
+template <class S>
+cudaError_t launch_seg_adjoint(const DevModel &M, int n_vch, const void *state_end,
+                               const void *info_incl, int se64, const float *pck,
+                               const float *segel, float *seg_info, float *seg_adj, int ck,
+                               int n_seg, cudaStream_t st) {
+  if (n_vch <= 0 || n_seg < 2) return cudaSuccess;
+  const int nb = (n_vch + 63) / 64;
+  k_seg_info<S><<<nb, 64, 0, st>>>(M, n_vch, info_incl, se64, segel, seg_info, ck);
+  GPSS_COUNT_LAUNCH();
+  k_seg_adjoint<S><<<dim3(nb, n_seg - 1), 64, 0, st>>>(M, n_vch, state_end, se64, pck, seg_info,
+                                                       seg_adj, ck);
   GPSS_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -2160,6 +2277,7 @@ OpTable make_ops() {
   o.plain64 = &launch_plain64<S>;
   o.elem = &launch_elem<S>;
   o.grad = &launch_grad<S>;
+  o.seg_adjoint = &launch_seg_adjoint<S>;
   o.disc = &launch_disc<S>;
   o.comb32 = make_combine<S, float>();
   o.tables = &launch_tables<S>;

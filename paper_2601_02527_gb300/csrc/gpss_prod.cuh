@@ -694,7 +694,7 @@ __global__ void __launch_bounds__(128) k_elem_prod(DevModel M, const float *__re
 template <bool SUM, class ES>
 cudaError_t launch_elem_prod(const DevModel &M, const float *theta, int n_vch, int per_series,
                              float *ef, double *ed, int *err, const float *, float *, int, float *,
-                             int c_begin, int c_count, cudaStream_t st) {
+                             int c_begin, int c_count, float *, int, cudaStream_t st) {
   if (n_vch <= 0 || c_count <= 0) return cudaSuccess;
   if (c_begin < 0 || c_begin + c_count > M.n_chunks) return cudaErrorInvalidValue;
   const int bs = 128;
