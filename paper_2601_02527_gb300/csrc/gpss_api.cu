@@ -270,6 +270,7 @@ struct gp_ss_model {
   int comb_prec = 32;      // arithmetic of the cross-chunk combination: 32 or 64
   int64_t *d_ch_ev0 = nullptr, *d_ch_meas0 = nullptr;
   int32_t *d_ch_len = nullptr, *d_ch_series = nullptr, *d_ch_first = nullptr;
+  int32_t *d_w_order = nullptr;  // warps of chunks, the longest chunks first
   std::vector<int32_t> ch_first;  // host copy: first chunk of each series
   uint8_t *d_ch_flags = nullptr;
   // step-scalar cache of the gradient: per warp of chunks, 32 x (its longest
@@ -378,7 +379,7 @@ void free_model_buffers(gp_ss_model *m) {
   void *dev[] = {m->d_ev_off, m->d_meas_off, m->d_dt, m->d_tag, m->d_meas, m->d_dt64, m->d_meas64,
                  m->d_mev,
                  m->d_ch_ev0, m->d_ch_meas0, m->d_ch_len, m->d_ch_series, m->d_ch_first,
-                 m->d_ch_flags, m->d_w_doff, m->d_err, m->d_ilv, m->d_ilv_tag};
+                 m->d_ch_flags, m->d_w_doff, m->d_w_order, m->d_err, m->d_ilv, m->d_ilv_tag};
   for (void *p : dev)
     if (p) cudaFree(p);
   if (m->pool) {
@@ -725,15 +726,20 @@ gp_ss_status make_plan(gp_ss_model *m, int chunk_len) {
   // every warp of 32 chunks lies in one series (32 | chunks per series)
   const size_t n_w = len.size() / 32;
   std::vector<int64_t> doff(n_w + 1, 0);
+  std::vector<int32_t> order(n_w);
   for (size_t w = 0; w < n_w; ++w) {
     int ml = 0;
     for (int l = 0; l < 32; ++l) ml = std::max(ml, len[w * 32 + l]);
     doff[w + 1] = doff[w] + 32 * (int64_t)ml;
+    order[w] = (int32_t)w;
   }
+  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+    return doff[x + 1] - doff[x] > doff[y + 1] - doff[y];
+  });
   // upload the new plan into fresh buffers first: the model keeps its old
   // plan, untouched, unless every upload succeeds
   int64_t *n_ev0 = nullptr, *n_meas0 = nullptr, *n_doff = nullptr;
-  int32_t *n_len = nullptr, *n_ser = nullptr, *n_first = nullptr;
+  int32_t *n_len = nullptr, *n_ser = nullptr, *n_first = nullptr, *n_order = nullptr;
   uint8_t *n_flags = nullptr;
   gp_ss_status st = GP_SS_OK;
   if (!st) st = dev_upload(&n_ev0, ev0.data(), ev0.size());
@@ -743,25 +749,28 @@ gp_ss_status make_plan(gp_ss_model *m, int chunk_len) {
   if (!st) st = dev_upload(&n_first, first.data(), first.size());
   if (!st) st = dev_upload(&n_flags, flags.data(), flags.size());
   if (!st) st = dev_upload(&n_doff, doff.data(), doff.size());
+  if (!st) st = dev_upload(&n_order, order.data(), order.size());
   // the event stream in this plan's lane-step order
   float4 *n_ilv = nullptr;
   uint8_t *n_ilv_tag = nullptr;
   if (!st) st = dev_upload<float4>(&n_ilv, nullptr, (size_t)doff[n_w]);
   if (!st) st = dev_upload<uint8_t>(&n_ilv_tag, nullptr, (size_t)doff[n_w]);
   if (st) {
-    void *fresh[] = {n_ev0, n_meas0, n_len, n_ser, n_first, n_flags, n_doff, n_ilv, n_ilv_tag};
+    void *fresh[] = {n_ev0,  n_meas0, n_len,   n_ser, n_first,
+                     n_flags, n_doff, n_order, n_ilv, n_ilv_tag};
     for (void *p : fresh)
       if (p) cudaFree(p);
     return st;
   }
   // kernels queued earlier may still read the old plan
   if (cudaDeviceSynchronize() != cudaSuccess) {
-    void *fresh[] = {n_ev0, n_meas0, n_len, n_ser, n_first, n_flags, n_doff, n_ilv, n_ilv_tag};
+    void *fresh[] = {n_ev0,  n_meas0, n_len,   n_ser, n_first,
+                     n_flags, n_doff, n_order, n_ilv, n_ilv_tag};
     for (void *p : fresh) cudaFree(p);
     return GP_SS_ECUDA;
   }
   void *old[] = {m->d_ch_ev0, m->d_ch_meas0, m->d_ch_len, m->d_ch_series, m->d_ch_first,
-                 m->d_ch_flags, m->d_w_doff, m->d_ilv, m->d_ilv_tag};
+                 m->d_ch_flags, m->d_w_doff, m->d_w_order, m->d_ilv, m->d_ilv_tag};
   for (void *p : old)
     if (p) cudaFree(p);
   m->d_ilv = n_ilv;
@@ -773,6 +782,7 @@ gp_ss_status make_plan(gp_ss_model *m, int chunk_len) {
   m->d_ch_first = n_first;
   m->d_ch_flags = n_flags;
   m->d_w_doff = n_doff;
+  m->d_w_order = n_order;
   m->ch_first = first;
   m->dcache_steps = doff[n_w];
   m->chunk_len = L;
@@ -811,6 +821,7 @@ gpss::DevModel dev_view(const gp_ss_model *m) {
   d.ch_first = m->d_ch_first;
   d.n_events = m->n_events;
   d.w_doff = m->d_w_doff;
+  d.w_order = m->d_w_order;
   d.dcache_steps = m->dcache_steps;
   d.ilv = m->d_ilv;
   d.ilv_tag = m->d_ilv_tag;

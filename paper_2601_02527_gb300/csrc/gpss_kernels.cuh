@@ -60,6 +60,7 @@ struct DevModel {
   const int32_t *ch_series;  // series of chunk
   const uint8_t *ch_flags;   // bit0 first chunk of its series, bit1 last
   const int32_t *ch_first;   // [n_series+1] first chunk of each series
+  const int32_t *w_order;    // warps of chunks, the longest chunks first
   // step-scalar cache layout: warp w of chunks (32 consecutive chunks, one
   // series) owns lane-steps [w_doff[w], w_doff[w+1]) of each theta set's
   // dcache_steps; the record of step k is DcW<NT>::G float4 groups x 32 lanes
@@ -76,6 +77,19 @@ struct DevModel {
   // every row then runs the kernels' general bodies, which read that bit
   int mixed;
 };
+
+// Chunk of parameter set `set` that thread l of a launch over all chunks of
+// n_vch / n_chunks sets works on: whole warps in the order of their chunks'
+// lengths, the longest first in every set, so that the last blocks to start
+// are the short ones (in the series' own order a long chunk could start when
+// the rest was done; 1024 series of 500 to 20000 exposures, 1.04 waves of
+// blocks: the element pass 407 -> 302 us, batch gradient of 1024 series: the
+// walk 1777 -> 1621 us).
+GPSS_D int chunk_of_thread(const DevModel &M, int n_vch, int l, int &set) {
+  const int n_sets = n_vch / M.n_chunks, w = l >> 5;
+  set = w % n_sets;
+  return M.w_order[w / n_sets] * 32 + (l & 31);
+}
 
 // Lane-step index of step k of chunk c.
 GPSS_D int64_t lane_step(const DevModel &M, int c, int k) {
@@ -627,8 +641,13 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
   // 32 chunks per series keeps each warp in one series)
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= (n_vch / M.n_chunks) * c_count) return;
-  const int set = l / c_count;
-  const int c = c_begin + l % c_count;
+  int set, c;
+  if (c_count == M.n_chunks) {
+    c = chunk_of_thread(M, n_vch, l, set);
+  } else {
+    set = l / c_count;
+    c = c_begin + l % c_count;
+  }
   const int vc = set * M.n_chunks + c;
   const int s = M.ch_series[c];
   const int row = per_series ? s : set;
@@ -1502,14 +1521,15 @@ __global__ void __launch_bounds__(GRAD_BS, GRAD_MIN_BLOCKS) k_grad(DevModel M, c
   constexpr int NDG = DcW<S::NT>::G;  // ... in float4 groups
   constexpr int SG = (SD + 3) / 4;    // replay slot: (m, P) in float4 groups
   extern __shared__ float sm[];
-  const int vc = blockIdx.x * blockDim.x + threadIdx.x;
-  if (vc >= n_vch) return;
+  const int vt = blockIdx.x * blockDim.x + threadIdx.x;
+  if (vt >= n_vch) return;
+  int set;
+  const int c = chunk_of_thread(M, n_vch, vt, set);
+  const int vc = set * M.n_chunks + c;
   // with seg_adj, this thread's only segment, counted from the chunk's end
   const int sq = blockIdx.y;
   rbuf += (size_t)sq * ck * (4 * SG) * n_vch;
   gpart += (size_t)sq * M.n_params * n_vch;
-  const int c = vc % M.n_chunks;
-  const int set = vc / M.n_chunks;
   const int s = M.ch_series[c];
   const int row = per_series ? s : set;
   const int orow = per_series ? s : set * M.n_series + s;
