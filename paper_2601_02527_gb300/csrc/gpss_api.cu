@@ -935,10 +935,88 @@ int grad_segments(const gp_ss_model *m, int n_vch, int ck) {
   return replay <= kMaxReplay ? n_seg : 1;
 }
 
+// Test times of a prediction, sorted and uploaded while the GPU runs the
+// element pass and the combination, which do not need them: enqueue calls
+// upload just before the gradient walk.  The host block and its device copy
+// hold off [n_events + n_series + 1], d [n_star] and idx [n_star] (PredPlan).
+struct PredJob {
+  const gp_ss_model *m;
+  const double *t_star;
+  const int64_t *star_offsets;
+  float *out;
+  std::vector<unsigned char> host;  // must outlive the copy
+  void *dev = nullptr;
+
+  // Each test time's interval: the first event at or after it (or none:
+  // after the series), gaps formed in FP64 and rounded once; then a counting
+  // sort, interior points by event, "after" points by series.  The search
+  // gallops from the previous test time's event, so ascending test times take
+  // a few comparisons each (13200 of them: the whole call 1073 -> 644 us
+  // with the upload behind the element pass).
+  gp_ss_status upload(gpss::PredPlan *pp, cudaStream_t st) {
+    const int ns = m->n_series;
+    const int64_t M = star_offsets[ns], nk = m->n_events + ns;
+    const size_t o_d = ((size_t)(nk + 2) * sizeof(int) + 15) & ~(size_t)15;
+    const size_t o_i = o_d + (size_t)M * sizeof(float2);
+    host.assign(o_i + (size_t)M * sizeof(int), 0);
+    // counts of key k go to cur[k + 2]; summed up, cur[k + 1] is the next place of
+    // key k and, once all are placed, the start of key k + 1
+    int *cur = reinterpret_cast<int *>(host.data());
+    float2 *d = reinterpret_cast<float2 *>(host.data() + o_d);
+    int *idx = reinterpret_cast<int *>(host.data() + o_i);
+    std::vector<int64_t> key(M);  // event index, or n_events + series for "after"
+    std::vector<float2> dd(M);
+    const double *t = m->tev.data();
+    for (int i = 0; i < ns; ++i) {
+      const int64_t e0 = m->ev_off[i], e1 = m->ev_off[i + 1];
+      int64_t k = e0;
+      for (int64_t j = star_offsets[i]; j < star_offsets[i + 1]; ++j) {
+        const double ts = t_star[j];
+        int64_t hi = k;
+        if (k > e0 && t[k - 1] >= ts) {  // before the previous test time's event
+          hi = k;
+          k = e0;
+        } else {
+          for (int64_t step = 1; hi < e1 && t[hi] < ts; step *= 2) {
+            k = hi + 1;
+            hi = std::min(e1, hi + step);
+          }
+        }
+        k = std::lower_bound(t + k, t + hi, ts) - t;
+        if (k == e1) {
+          key[j] = m->n_events + i;
+          dd[j] = make_float2((float)(ts - t[e1 - 1]), 0.f);
+        } else {
+          key[j] = k;
+          dd[j] = make_float2(k == e0 ? 0.f : (float)(ts - t[k - 1]), (float)(t[k] - ts));
+        }
+        ++cur[key[j] + 2];
+      }
+    }
+    for (int64_t k = 0; k < nk; ++k) cur[k + 1] += cur[k];
+    for (int64_t j = 0; j < M; ++j) {
+      const int at = cur[key[j] + 1]++;
+      idx[at] = (int)j;
+      d[at] = dd[j];
+    }
+    if (scratch_alloc(m, &dev, host.size(), st) != cudaSuccess) return GP_SS_ENOMEM;
+    if (cudaMemcpyAsync(dev, host.data(), host.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
+      return GP_SS_ECUDA;
+    unsigned char *b = static_cast<unsigned char *>(dev);
+    pp->off = reinterpret_cast<int *>(b);
+    pp->xoff = pp->off + m->n_events;
+    pp->d = reinterpret_cast<float2 *>(b + o_d);
+    pp->idx = reinterpret_cast<int *>(b + o_i);
+    pp->out = out;
+    pp->n_star = M;
+    return GP_SS_OK;
+  }
+};
+
 // Enqueue the log-likelihood (and optionally gradient) computation.
 gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int per_series,
                      double *ll, float *grad, cudaStream_t st, float *dexp = nullptr,
-                     float *cond_out = nullptr, const gpss::PredPlan *pred = nullptr,
+                     float *cond_out = nullptr, PredJob *pred = nullptr,
                      const ElemSlices *slices = nullptr) {
   const int n_out = per_series ? m->n_series : n_sets * m->n_series;
   gp_ss_status s0 = prepare_err(m, n_out, st);
@@ -1134,12 +1212,13 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
           res = GP_SS_ECUDA;
         if (res) break;
       } else {
-        const gpss::PredPlan none;
+        gpss::PredPlan pp;
+        if (pred && (res = pred->upload(&pp, st))) break;
         n_gpart = n_seg;
         if ((n_seg > 1 && o.seg_adjoint(dm, n_vch, state_end, info, eb == 8 ? 1 : 0, ckpt, segel,
                                         seg_info, seg_adj, ck, n_seg, st)) ||
             o.grad(dm, theta, n_vch, per_series, state_end, eb == 8 ? 1 : 0, adj, ckpt, gpart,
-                   m->d_err, tabs, rbuf, dcache, ck, gdt, gwe, cond, pred ? *pred : none,
+                   m->d_err, tabs, rbuf, dcache, ck, gdt, gwe, cond, pp,
                    seg_adj, n_seg, st)) {
           res = GP_SS_ECUDA;
           break;
@@ -1556,77 +1635,21 @@ gp_ss_status gp_ss_predict(const gp_ss_model *m, const float *theta, int n_sets,
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const int n_out = theta_per_series ? m->n_series : n_sets * m->n_series;
   if (M == 0) return gp_ss_loglik(m, theta, n_sets, theta_per_series, loglik_out, cuda_stream);
-  // each test time's interval: the first event at or after it (or none: after
-  // the series); gaps formed in FP64 and rounded once
-  std::vector<int64_t> key(M);  // event index, or n_events + series for "after"
-  std::vector<float2> dd(M);
-  std::vector<int> cnt(m->n_events + ns + 1, 0);
-  for (int i = 0; i < ns; ++i) {
-    const int64_t e0 = m->ev_off[i], e1 = m->ev_off[i + 1];
-    const double *t = m->tev.data();
-    for (int64_t j = star_offsets[i]; j < star_offsets[i + 1]; ++j) {
-      const double ts = t_star[j];
-      const int64_t k = std::lower_bound(t + e0, t + e1, ts) - t;
-      if (e1 == e0) {
-        key[j] = m->n_events + i;  // empty series: the prior (no data)
-        dd[j] = make_float2(0.f, 0.f);
-      } else if (k == e1) {
-        key[j] = m->n_events + i;
-        dd[j] = make_float2((float)(ts - t[e1 - 1]), 0.f);
-      } else if (k == e0) {
-        key[j] = k;
-        dd[j] = make_float2(0.f, (float)(t[k] - ts));
-      } else {
-        key[j] = k;
-        dd[j] = make_float2((float)(ts - t[k - 1]), (float)(t[k] - ts));
-      }
-      ++cnt[key[j]];
-    }
-  }
-  // counting sort by key: interior points by event, then "after" points by series
-  std::vector<int> off(m->n_events + ns + 1, 0);
-  for (int64_t k = 0; k < m->n_events + ns; ++k) off[k + 1] = off[k] + cnt[k];
-  std::vector<int> pos(off.begin(), off.end() - 1), idx(M);
-  std::vector<float2> dsort(M);
-  for (int64_t j = 0; j < M; ++j) {
-    const int p = pos[key[j]]++;
-    idx[p] = (int)j;
-    dsort[p] = dd[j];
-  }
-  gp_ss_status res = GP_SS_OK;
-  int *d_off = nullptr, *d_idx = nullptr;
-  float2 *d_d = nullptr;
+  // points of empty series would need the prior, which no kernel visits
+  for (int i = 0; i < ns; ++i)
+    if (m->ev_off[i] == m->ev_off[i + 1] && star_offsets[i + 1] > star_offsets[i])
+      return GP_SS_EUNSUPPORTED;
+  PredJob job{m, t_star, star_offsets, pred_out, {}, nullptr};
   float *grad = nullptr;
-  const size_t noff = off.size();
-  if (scratch_alloc(m, (void **)&d_off, noff * sizeof(int), st) ||
-      scratch_alloc(m, (void **)&d_idx, M * sizeof(int), st) ||
-      scratch_alloc(m, (void **)&d_d, M * sizeof(float2), st) ||
-      scratch_alloc(m, (void **)&grad, (size_t)n_out * m->n_params * sizeof(float), st))
+  gp_ss_status res = GP_SS_OK;
+  if (scratch_alloc(m, (void **)&grad, (size_t)n_out * m->n_params * sizeof(float), st) !=
+      cudaSuccess)
     res = GP_SS_ENOMEM;
-  if (!res && (cudaMemcpyAsync(d_off, off.data(), noff * sizeof(int), cudaMemcpyHostToDevice, st) ||
-               cudaMemcpyAsync(d_idx, idx.data(), M * sizeof(int), cudaMemcpyHostToDevice, st) ||
-               cudaMemcpyAsync(d_d, dsort.data(), M * sizeof(float2), cudaMemcpyHostToDevice, st)))
-    res = GP_SS_ECUDA;
-  // points of empty series: the prior, which no kernel visits
-  if (!res) {
-    bool any_empty = false;
-    for (int i = 0; i < ns; ++i) any_empty |= (m->ev_off[i] == m->ev_off[i + 1] &&
-                                               star_offsets[i + 1] > star_offsets[i]);
-    if (any_empty) res = GP_SS_EUNSUPPORTED;
-  }
-  if (!res) {
-    gpss::PredPlan pp;
-    pp.off = d_off;
-    pp.xoff = d_off + m->n_events;
-    pp.idx = d_idx;
-    pp.d = d_d;
-    pp.out = pred_out;
-    pp.n_star = M;
-    res = enqueue(m, theta, n_sets, theta_per_series, loglik_out, grad, st, nullptr, nullptr, &pp);
-  }
-  // the host vectors must outlive the copies
+  if (!res)
+    res = enqueue(m, theta, n_sets, theta_per_series, loglik_out, grad, st, nullptr, nullptr, &job);
+  // the host block must outlive the copy
   if (cudaStreamSynchronize(st) != cudaSuccess && !res) res = GP_SS_ECUDA;
-  for (void *p : {(void *)d_off, (void *)d_idx, (void *)d_d, (void *)grad})
+  for (void *p : {job.dev, (void *)grad})
     if (p) cudaFreeAsync(p, st);
   return res;
 }
