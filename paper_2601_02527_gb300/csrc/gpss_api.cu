@@ -1126,8 +1126,27 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
         n_seg = 1;
       }
     }
+    // product models: the oscillators' scalars of every step (the gradient's
+    // with their tangents), within the same bound and where the memory is there
+    float *ptan = nullptr;
+    if (m->product && m->step_cache == 0 && m->max_chunk <= 65535 * gpss::PROD_STEPS) {
+      const size_t bytes =
+          (size_t)(n_vch / m->n_chunks) * (size_t)m->dcache_steps * (o.D / 2) * sizeof(float4);
+      if (bytes * (grad ? 3 : 1) <= kDcacheMax && grab((void **)&dcache, bytes) && grad &&
+          !grab((void **)&ptan, 2 * bytes)) {
+        cudaFreeAsync(dcache, st);
+        bufs.pop_back();
+        dcache = nullptr;
+      }
+      cudaGetLastError();
+    }
     {
       PhaseTimer pt(m, st, 0);
+      if (m->product && dcache &&
+          o.prod_scalars(dm, theta, n_vch, per_series, m->max_chunk, dcache, ptan, st)) {
+        res = GP_SS_ECUDA;
+        break;
+      }
       if (o.tables(theta, n_sets, m->n_params, m->kinds[0], m->kinds[1], tabs, st)) {
         res = GP_SS_ECUDA;
         break;
@@ -1208,7 +1227,7 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
       if (m->product) {
         // chunked forward-mode tangents against the boundary adjoints
         if (o.prod_grad_chunk(dm, theta, n_vch, per_series, state_end, eb == 8 ? 1 : 0, adj, gpart,
-                              m->d_err, st))
+                              m->d_err, dcache, ptan, st))
           res = GP_SS_ECUDA;
         if (res) break;
       } else {

@@ -2035,6 +2035,8 @@ cudaError_t launch_span_fold(const double *elems, int n_spans, int n_rows, doubl
 // ---------------------------------------------------------------------------
 // Host launchers, one table per compiled shape.
 // ---------------------------------------------------------------------------
+constexpr int PROD_STEPS = 8;  // steps per block of a product model's k_prod_scalars
+
 // Cross-chunk combination in one arithmetic (FP32 or FP64): the sequential
 // fold per series, the warp-level scans with the scan or fold of warp totals
 // and the per-chunk join, and the chunk log-likelihoods with the boundary
@@ -2079,7 +2081,12 @@ struct OpTable {
   // product models, chunked schedule: gradient parts per (chunk, parameter)
   // from the combination's incoming states and boundary adjoints (else null)
   cudaError_t (*prod_grad_chunk)(const DevModel &, const float *, int, int, const void *, int,
-                                 const float *, float *, int *, cudaStream_t);
+                                 const float *, float *, int *, const float *, const float *,
+                                 cudaStream_t);
+  // product models: the oscillators' step scalars (and tangents) of all steps,
+  // given the longest chunk (else null)
+  cudaError_t (*prod_scalars)(const DevModel &, const float *, int, int, int, float *, float *,
+                              cudaStream_t);
   // a series split in time: element of a chunk range, fold of span elements
   cudaError_t (*span_element)(const float *, const double *, int, int, int, int, int, double *,
                               double *, cudaStream_t);

@@ -33,11 +33,15 @@ struct Osc2 {
 };
 
 template <class T, class F>
-GPSS_HD Osc2<T> osc2(F dt, T w0, T Q, T var) {
-  const T a = w0 / (F(2) * Q);
-  const T beta = (val(Q) == F(0.5)) ? cst<T>(F(0))
-                                    : w0 * w0 * (F(1) - cst<T>(F(1)) / (F(4) * Q * Q));
-  const Disc<T> d = discretize<T, F, true>(dt, a, beta);
+GPSS_HD void osc_rates(T w0, T Q, T &a, T &beta) {
+  a = w0 / (F(2) * Q);
+  beta = (val(Q) == F(0.5)) ? cst<T>(F(0))
+                            : w0 * w0 * (F(1) - cst<T>(F(1)) / (F(4) * Q * Q));
+}
+
+// From the step's scalars d (f, f', I_ff and I_pp are read).
+template <class T, class F>
+GPSS_HD Osc2<T> osc2_of(const Disc<T> &d, T a, T w0, T Q, T var) {
   const T qc = F(2) * w0 * w0 * w0 * var / Q;
   Osc2<T> o;
   o.p[0][0] = d.fp + F(2) * a * d.f;
@@ -48,6 +52,124 @@ GPSS_HD Osc2<T> osc2(F dt, T w0, T Q, T var) {
   o.q[0][1] = o.q[1][0] = qc * d.f * d.f * F(0.5);
   o.q[1][1] = qc * d.Ipp;
   return o;
+}
+
+template <class T, class F>
+GPSS_HD Osc2<T> osc2(F dt, T w0, T Q, T var) {
+  T a, beta;
+  osc_rates<T, F>(w0, Q, a, beta);
+  return osc2_of<T, F>(discretize<T, F, true>(dt, a, beta), a, w0, Q, var);
+}
+
+// ---------------------------------------------------------------------------
+// Step scalars of a product model's oscillators, formed for all steps at once
+// before the chunk kernels: they depend on no other step, and a Taylor double
+// sum per oscillator was most of a chunk's serial chain (and, as duals, of
+// every parameter's thread in the gradient).  Per lane-step and oscillator
+// one float4 (f, f', I_ff, I_pp), oscillator j of step k of the chunk on lane
+// l of warp w at ((w_doff[w] + 32 k) NO + 32 j + l); with tangents, two more
+// float4 (d/da, d/dbeta of the four) behind all sets' values, in the same
+// order.  150 series of 500 to 5000 instants with the gradient, product +
+// Matern-3/2: scalars 67 us, elements 442 -> 121 us, gradient 1099 -> 304 us.
+// ---------------------------------------------------------------------------
+template <bool SUM>
+struct ProdOsc {
+  static constexpr int NO = SUM ? 3 : 2;
+};
+
+// Rates of oscillator j of a parameter row.
+template <bool SUM>
+GPSS_HD void prod_osc(const DevModel &M, const float *th, int j, float &w0, float &Q) {
+  if (j < 2) {
+    w0 = th[1 + 2 * j];
+    Q = th[2 + 2 * j];
+  } else if (M.kinds[1] == 1) {
+    w0 = th[6];
+    Q = th[7];
+  } else {
+    w0 = float(1.7320508075688772) / th[6];
+    Q = 0.5f;
+  }
+}
+
+// Whether a parameter row has an overdamped factor or plain term.
+template <bool SUM>
+GPSS_D bool prod_overdamped(const DevModel &M, const float *th) {
+  return th[2] < 0.5f || th[4] < 0.5f || (SUM && M.kinds[1] == 1 && th[7] < 0.5f);
+}
+
+GPSS_D size_t prod_col(const DevModel &M, int set, int c) {
+  return (size_t)set * M.dcache_steps + M.w_doff[c >> 5];
+}
+
+template <bool SUM>
+__global__ void __launch_bounds__(128) k_prod_scalars(DevModel M, const float *__restrict__ theta,
+                                                      int n_vch, int per_series,
+                                                      float4 *__restrict__ sc,
+                                                      float4 *__restrict__ tan) {
+  using F = float;
+  constexpr int NO = ProdOsc<SUM>::NO;
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l >= n_vch) return;
+  const int set = l / M.n_chunks, c = l % M.n_chunks, j = blockIdx.z, lane = c & 31;
+  const int k0 = blockIdx.y * PROD_STEPS, k1 = min(M.ch_len[c], k0 + PROD_STEPS);
+  if (k0 >= k1) return;
+  F w0, Q, a, beta;
+  prod_osc<SUM>(M, theta + (size_t)(per_series ? M.ch_series[c] : set) * M.n_params, j, w0, Q);
+  osc_rates<F, F>(w0, Q, a, beta);
+  const size_t col = prod_col(M, set, c);
+  for (int k = k0; k < k1; ++k) {
+    const F dt = __ldg(M.ilv + lane_step(M, c, k)).x;
+    const Disc<F> d = discretize<F, F, true>(dt, a, beta);
+    const size_t at = (col + (size_t)k * 32) * NO + 32 * j + lane;
+    sc[at] = make_float4(d.f, d.fp, d.Iff, d.Ipp);
+    if (tan) {
+      using T = Dual2<F>;
+      const Disc<T> e = discretize<T, F, true>(dt, mk(a, F(1), F(0)), mk(beta, F(0), F(1)));
+      const size_t t0 = (col + (size_t)k * 32) * (2 * NO) + 64 * j + lane;
+      tan[t0] = make_float4(e.f.da, e.fp.da, e.Iff.da, e.Ipp.da);
+      tan[t0 + 32] = make_float4(e.f.db, e.fp.db, e.Iff.db, e.Ipp.db);
+    }
+  }
+}
+
+// Values of oscillator j at a step's record (the first of its NO float4 rows).
+GPSS_D Disc<float> prod_load(const float4 *rec, int j) {
+  const float4 q = __ldg(rec + 32 * j);
+  Disc<float> d;
+  d.f = q.x;
+  d.fp = q.y;
+  d.Iff = q.z;
+  d.Ipp = q.w;
+  d.F1 = d.IFF = 0.f;
+  return d;
+}
+
+// ... with the tangent of the thread's parameter, (a.da, beta.da).
+GPSS_D Disc<Dual2<float>> prod_load_dual(const float4 *rec, const float4 *trec, int j, float da,
+                                         float db) {
+  const float4 q = __ldg(rec + 32 * j), ta = __ldg(trec + 64 * j), tb = __ldg(trec + 64 * j + 32);
+  Disc<Dual2<float>> d;
+  d.f = mk(q.x, ta.x * da + tb.x * db, 0.f);
+  d.fp = mk(q.y, ta.y * da + tb.y * db, 0.f);
+  d.Iff = mk(q.z, ta.z * da + tb.z * db, 0.f);
+  d.Ipp = mk(q.w, ta.w * da + tb.w * db, 0.f);
+  d.F1 = d.IFF = mk(0.f, 0.f, 0.f);
+  return d;
+}
+
+template <bool SUM>
+cudaError_t launch_prod_scalars(const DevModel &M, const float *theta, int n_vch, int per_series,
+                                int max_len, float *sc, float *tan, cudaStream_t st) {
+  if (n_vch <= 0 || max_len <= 0) return cudaSuccess;
+  const dim3 nb((unsigned)((n_vch + 127) / 128), (unsigned)((max_len + PROD_STEPS - 1) / PROD_STEPS),
+                ProdOsc<SUM>::NO);
+  if (nb.y > 65535) return cudaErrorInvalidValue;
+  k_prod_scalars<SUM><<<nb, 128, 0, st>>>(M, theta, n_vch, per_series,
+                                          reinterpret_cast<float4 *>(sc),
+                                          reinterpret_cast<float4 *>(tan));
+  GPSS_COUNT_LAUNCH();
+  return cudaGetLastError();
 }
 
 // One thread per (parameter set, series).  Parameter row: (sigma, omega_a,
@@ -267,16 +389,21 @@ GPSS_D void prod_prior(const ProdPar<SUM> &p, Dual2<float> (*m), Dual2<float> (*
 
 // One event (instantaneous measurement y with variance r0) of the dual
 // product filter on the dense (m, P); adds log S + v^2/S and its tangent.
+//
+// Phi is block-diagonal (the product's Kronecker block, then the plain term):
+// the sums run over the blocks only.  The tangent's terms use S's reciprocal,
+// the FP32 one refined by a Newton step in FP64 (error 1e-14), in place of
+// three FP64 divisions, which took most of an event's time.
 template <bool SUM>
-GPSS_D void prod_event(const ProdPar<SUM> &p, float dt, float y, float r0, Dual2<float> *m,
-                       Dual2<float> (*P)[SUM ? 6 : 4], double &sum_ll, double &sum_d, bool &bad) {
+GPSS_D void prod_event(const ProdPar<SUM> &p, const Osc2<Dual2<float>> &A,
+                       const Osc2<Dual2<float>> &B, const Osc2<Dual2<float>> &C, float y, float r0,
+                       Dual2<float> *m, Dual2<float> (*P)[SUM ? 6 : 4], double &sum_ll,
+                       double &sum_d, bool &bad) {
   using F = float;
   using T = Dual2<F>;
   constexpr int D = SUM ? 6 : 4;
   const T one = cst<T>(F(1));
   const T Pa[2] = {one, p.wa * p.wa}, Pb[2] = {p.var, p.var * p.wb * p.wb};
-  const Osc2<T> A = osc2<T, F>(dt, p.wa, p.qa, one);
-  const Osc2<T> B = osc2<T, F>(dt, p.wb, p.qb, p.var);
   T Phi[D][D], Qd[D][D];
 #pragma unroll
   for (int r = 0; r < D; ++r)
@@ -298,7 +425,6 @@ GPSS_D void prod_event(const ProdPar<SUM> &p, float dt, float y, float r0, Dual2
           Qd[r][c] = q;
         }
   if constexpr (SUM) {
-    const Osc2<T> C = osc2<T, F>(dt, p.wc, p.qcq, p.sc * p.sc);
 #pragma unroll
     for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -310,15 +436,16 @@ GPSS_D void prod_event(const ProdPar<SUM> &p, float dt, float y, float r0, Dual2
   T mt[D], Tm[D][D];
 #pragma unroll
   for (int r = 0; r < D; ++r) {
+    const int b0 = r < 4 ? 0 : 4, b1 = r < 4 ? 4 : D;  // the row's block
     T acc = cst<T>(F(0));
 #pragma unroll
-    for (int c = 0; c < D; ++c) acc = acc + Phi[r][c] * m[c];
+    for (int c = b0; c < b1; ++c) acc = acc + Phi[r][c] * m[c];
     mt[r] = acc;
 #pragma unroll
     for (int c = 0; c < D; ++c) {
       T a2 = cst<T>(F(0));
 #pragma unroll
-      for (int e = 0; e < D; ++e) a2 = a2 + Phi[r][e] * P[e][c];
+      for (int e = b0; e < b1; ++e) a2 = a2 + Phi[r][e] * P[e][c];
       Tm[r][c] = a2;
     }
   }
@@ -327,9 +454,10 @@ GPSS_D void prod_event(const ProdPar<SUM> &p, float dt, float y, float r0, Dual2
     m[r] = mt[r];
 #pragma unroll
     for (int c = r; c < D; ++c) {
+      const int b0 = c < 4 ? 0 : 4, b1 = c < 4 ? 4 : D;
       T a2 = Qd[r][c];
 #pragma unroll
-      for (int e = 0; e < D; ++e) a2 = a2 + Tm[r][e] * Phi[c][e];
+      for (int e = b0; e < b1; ++e) a2 = a2 + Tm[r][e] * Phi[c][e];
       P[r][c] = a2;
       P[c][r] = a2;
     }
@@ -350,8 +478,10 @@ GPSS_D void prod_event(const ProdPar<SUM> &p, float dt, float y, float r0, Dual2
     for (int c = 0; c < D; ++c) P[r][c] = P[r][c] - u[r] * u[c] * iS;
   }
   const double S = Sv.v, dS = Sv.da, e = vv.v, de = vv.da;
-  sum_ll += log(S) + e * e / S;
-  sum_d += dS / S + 2.0 * e * de / S - e * e * dS / (S * S);
+  double iSd = iS.v;
+  iSd = iSd * (2.0 - S * iSd);
+  sum_ll += log(S) + e * e * iSd;
+  sum_d += iSd * (dS * (1.0 - e * e * iSd) + 2.0 * e * de);
 }
 
 // One thread per (output row, parameter i) over the whole series (the plain
@@ -383,7 +513,12 @@ __global__ void __launch_bounds__(64) k_prod_grad(DevModel M, const float *__res
     F y, r0, w;
     load_meas<F>(M, mi, y, r0, w);
     ++mi;
-    prod_event<SUM>(p, load_dt<F>(M, k), y, r0, m, P, sum_ll, sum_d, bad);
+    const F dt = load_dt<F>(M, k);
+    const Osc2<T> A = osc2<T, F>(dt, p.wa, p.qa, cst<T>(F(1)));
+    const Osc2<T> B = osc2<T, F>(dt, p.wb, p.qb, p.var);
+    Osc2<T> C{};
+    if constexpr (SUM) C = osc2<T, F>(dt, p.wc, p.qcq, p.sc * p.sc);
+    prod_event<SUM>(p, A, B, C, y, r0, m, P, sum_ll, sum_d, bad);
     ++n_end;
   }
   const double ll = -0.5 * ((double)n_end * LOG_2PI + sum_ll);
@@ -412,10 +547,12 @@ __global__ void __launch_bounds__(64) k_prod_grad_chunk(DevModel M, const float 
                                                         const void *__restrict__ state_end, int se64,
                                                         const float *__restrict__ adj_end,
                                                         float *__restrict__ gpart,
-                                                        int *__restrict__ err) {
+                                                        int *__restrict__ err,
+                                                        const float4 *__restrict__ sc,
+                                                        const float4 *__restrict__ tan) {
   using F = float;
   using T = Dual2<F>;
-  constexpr int D = SUM ? 6 : 4;
+  constexpr int D = SUM ? 6 : 4, NO = ProdOsc<SUM>::NO;
   static_assert(ES::D == D, "combination shape of the product's state size");
   const int np = M.n_params;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -443,13 +580,32 @@ __global__ void __launch_bounds__(64) k_prod_grad_chunk(DevModel M, const float 
   }
   double sum_ll = 0.0, sum_d = 0.0;
   bool bad = false;
-  int64_t mi = M.ch_meas0[c];
-  const int64_t k0 = M.ch_ev0[c], k1 = k0 + M.ch_len[c];
-  for (int64_t k = k0; k < k1; ++k) {
-    F y, r0, w;
-    load_meas<F>(M, mi, y, r0, w);
-    ++mi;
-    prod_event<SUM>(p, load_dt<F>(M, k), y, r0, m, P, sum_ll, sum_d, bad);
+  // the oscillators' rates with their tangents, and the step records
+  T aa, ba, ab, bb, ac, bc;
+  osc_rates<T, F>(p.wa, p.qa, aa, ba);
+  osc_rates<T, F>(p.wb, p.qb, ab, bb);
+  osc_rates<T, F>(p.wc, p.qcq, ac, bc);
+  const T one = cst<T>(F(1)), varc = p.sc * p.sc;
+  const size_t col = prod_col(M, set, c);
+  const float4 *rec = sc ? sc + col * NO + (c & 31) : nullptr;
+  const float4 *trec = sc ? tan + col * (2 * NO) + (c & 31) : nullptr;
+  const int len = M.ch_len[c];
+  for (int k = 0; k < len; ++k) {
+    const float4 q = __ldg(M.ilv + lane_step(M, c, k));  // (dt, y, yerr^2, 1)
+    Osc2<T> A, B, C{};
+    if (rec) {
+      A = osc2_of<T, F>(prod_load_dual(rec, trec, 0, aa.da, ba.da), aa, p.wa, p.qa, one);
+      B = osc2_of<T, F>(prod_load_dual(rec, trec, 1, ab.da, bb.da), ab, p.wb, p.qb, p.var);
+      if constexpr (SUM)
+        C = osc2_of<T, F>(prod_load_dual(rec, trec, 2, ac.da, bc.da), ac, p.wc, p.qcq, varc);
+      rec += 32 * NO;
+      trec += 64 * NO;
+    } else {
+      A = osc2<T, F>(q.x, p.wa, p.qa, one);
+      B = osc2<T, F>(q.x, p.wb, p.qb, p.var);
+      if constexpr (SUM) C = osc2<T, F>(q.x, p.wc, p.qcq, varc);
+    }
+    prod_event<SUM>(p, A, B, C, q.y, q.z, m, P, sum_ll, sum_d, bad);
   }
   double g = -0.5 * sum_d;
   if (!(flags & 2)) {
@@ -483,12 +639,14 @@ cudaError_t launch_prod_grad(const DevModel &M, const float *theta, int n_out, i
 template <bool SUM, class ES>
 cudaError_t launch_prod_grad_chunk(const DevModel &M, const float *theta, int n_vch, int per_series,
                                    const void *state_end, int se64, const float *adj_end,
-                                   float *gpart, int *err, cudaStream_t st) {
+                                   float *gpart, int *err, const float *sc, const float *tan,
+                                   cudaStream_t st) {
   if (n_vch <= 0) return cudaSuccess;
   const int bs = 64;
   const int64_t nt = (int64_t)n_vch * M.n_params;
   k_prod_grad_chunk<SUM, ES><<<(unsigned)((nt + bs - 1) / bs), bs, 0, st>>>(
-      M, theta, n_vch, per_series, state_end, se64, adj_end, gpart, err);
+      M, theta, n_vch, per_series, state_end, se64, adj_end, gpart, err, reinterpret_cast<const float4 *>(sc),
+      reinterpret_cast<const float4 *>(tan));
   GPSS_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -514,19 +672,25 @@ __global__ void __launch_bounds__(128) k_elem_prod(DevModel M, const float *__re
                                                    int n_vch, int per_series,
                                                    float *__restrict__ ef, double *__restrict__ ed,
                                                    int *__restrict__ err, int c_begin,
-                                                   int c_count) {
+                                                   int c_count, int od_only) {
   using F = float;
   constexpr int D = SUM ? 6 : 4;
   static_assert(ES::D == D, "element shape of the product state");
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= (n_vch / M.n_chunks) * c_count) return;
-  const int set = l / c_count;
-  const int c = c_begin + l % c_count;
+  int set, c;
+  if (c_count == M.n_chunks) {
+    c = chunk_of_thread(M, n_vch, l, set);
+  } else {
+    set = l / c_count;
+    c = c_begin + l % c_count;
+  }
   const int vc = set * M.n_chunks + c;
   const int s = M.ch_series[c];
   const int row = per_series ? s : set;
   const int orow = per_series ? s : set * M.n_series + s;
   const float *th = theta + (size_t)row * M.n_params;
+  if (od_only && !prod_overdamped<SUM>(M, th)) return;
   const F sig = th[0], wa = th[1], qa = th[2], wb = th[3], qb = th[4];
   const F var = sig * sig;
   const F Pa[2] = {F(1), wa * wa}, Pb[2] = {var, var * wb * wb};
@@ -691,16 +855,221 @@ __global__ void __launch_bounds__(128) k_elem_prod(DevModel M, const float *__re
   if (bad) flag_error(err, orow, 7);
 }
 
+// The same from precomputed scalars (k_prod_scalars), for the rows without an
+// overdamped factor: the same FP32 operations on them, so the same bits.  Rows
+// with an overdamped factor stay with k_elem_prod (a second launch that skips
+// the others): the doubling of their integrals rounds differently once it is
+// compiled into another kernel, by 1e-8 of the log-likelihood.
+template <bool SUM, class ES>
+__global__ void __launch_bounds__(128) k_elem_prod_pre(DevModel M,
+                                                       const float *__restrict__ theta, int n_vch,
+                                                       int per_series, float *__restrict__ ef,
+                                                       double *__restrict__ ed,
+                                                       int *__restrict__ err, int c_begin,
+                                                       int c_count, const float4 *__restrict__ sc) {
+  using F = float;
+  constexpr int D = SUM ? 6 : 4, NO = ProdOsc<SUM>::NO;
+  static_assert(ES::D == D, "element shape of the product state");
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l >= (n_vch / M.n_chunks) * c_count) return;
+  int set, c;
+  if (c_count == M.n_chunks) {
+    c = chunk_of_thread(M, n_vch, l, set);
+  } else {
+    set = l / c_count;
+    c = c_begin + l % c_count;
+  }
+  const int vc = set * M.n_chunks + c;
+  const int s = M.ch_series[c];
+  const int row = per_series ? s : set;
+  const int orow = per_series ? s : set * M.n_series + s;
+  const float *th = theta + (size_t)row * M.n_params;
+  if (prod_overdamped<SUM>(M, th)) return;
+  const F sig = th[0], wa = th[1], qa = th[2], wb = th[3], qb = th[4];
+  const F var = sig * sig;
+  const F Pa[2] = {F(1), wa * wa}, Pb[2] = {var, var * wb * wb};
+  F sgc = F(0), wc = F(1), qcq = F(0.5);
+  int j = 5;
+  if constexpr (SUM) {
+    sgc = th[5];
+    if (M.kinds[1] == 1) {
+      wc = th[6];
+      qcq = th[7];
+      j = 8;
+    } else {
+      wc = F(1.7320508075688772) / F(th[6]);
+      j = 7;
+    }
+  }
+  const F s2 = F(th[j]) * F(th[j]);
+  const bool first = M.ch_flags[c] & 1;
+  // element: A (D x D), b, C (full here, packed on store), eta, J (full)
+  F A[D][D], b[D], C[D][D], eta[D], J[D][D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    b[i] = F(0);
+    eta[i] = F(0);
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      A[i][k] = (!first && i == k) ? F(1) : F(0);
+      C[i][k] = F(0);
+      J[i][k] = F(0);
+    }
+  }
+  if (first) {  // the series' first chunk starts from the prior
+#pragma unroll
+    for (int ra = 0; ra < 2; ++ra)
+#pragma unroll
+      for (int rb = 0; rb < 2; ++rb) C[2 * ra + rb][2 * ra + rb] = Pa[ra] * Pb[rb];
+    if constexpr (SUM) {
+      C[4][4] = sgc * sgc;
+      C[5][5] = sgc * sgc * wc * wc;
+    }
+  }
+  double gam = 0.0, ld = 0.0;
+  int n_end = 0;
+  bool bad = false;
+  const int len = M.ch_len[c];
+  const F aa = wa / (F(2) * qa), ab = wb / (F(2) * qb), ac = wc / (F(2) * qcq);
+  const float4 *rec = sc + prod_col(M, set, c) * NO + (c & 31);
+  for (int kk = 0; kk < len; ++kk) {
+    const float4 q = __ldg(M.ilv + lane_step(M, c, kk));  // (dt, y, yerr^2, 1)
+    const Disc<F> da = prod_load(rec, 0), db = prod_load(rec, 1);
+    const Osc2<F> Ao = osc2_of<F, F>(da, aa, wa, qa, F(1));
+    const Osc2<F> Bo = osc2_of<F, F>(db, ab, wb, qb, var);
+    F Phi[D][D], Qd[D][D];
+#pragma unroll
+    for (int r = 0; r < D; ++r)
+#pragma unroll
+      for (int cc = 0; cc < D; ++cc) Phi[r][cc] = Qd[r][cc] = F(0);
+#pragma unroll
+    for (int ra = 0; ra < 2; ++ra)
+#pragma unroll
+      for (int rb = 0; rb < 2; ++rb)
+#pragma unroll
+        for (int ca = 0; ca < 2; ++ca)
+#pragma unroll
+          for (int cb = 0; cb < 2; ++cb) {
+            const int r = 2 * ra + rb, cc = 2 * ca + cb;
+            Phi[r][cc] = Ao.p[ra][ca] * Bo.p[rb][cb];
+            Qd[r][cc] = (ra == ca ? Pa[ra] * Bo.q[rb][cb] : F(0)) +
+                        (rb == cb ? Ao.q[ra][ca] * Pb[rb] : F(0)) - Ao.q[ra][ca] * Bo.q[rb][cb];
+          }
+    if constexpr (SUM) {
+      const Osc2<F> Co = osc2_of<F, F>(prod_load(rec, 2), ac, wc, qcq, sgc * sgc);
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+          Phi[4 + r][4 + cc] = Co.p[r][cc];
+          Qd[4 + r][4 + cc] = Co.q[r][cc];
+        }
+    }
+    rec += 32 * NO;
+    // A <- Phi A, b <- Phi b, C <- Phi C Phi^T + Q; Phi is block-diagonal, and
+    // the sums run over the row's block (the rest would add zeros)
+    F T1[D][D], T2[D][D], bt[D];
+#pragma unroll
+    for (int r = 0; r < D; ++r) {
+      const int b0 = r < 4 ? 0 : 4, b1 = r < 4 ? 4 : D;
+      F acc = F(0);
+#pragma unroll
+      for (int e = b0; e < b1; ++e) acc += Phi[r][e] * b[e];
+      bt[r] = acc;
+#pragma unroll
+      for (int cc = 0; cc < D; ++cc) {
+        F a1 = F(0), a2 = F(0);
+#pragma unroll
+        for (int e = b0; e < b1; ++e) {
+          a1 += Phi[r][e] * A[e][cc];
+          a2 += Phi[r][e] * C[e][cc];
+        }
+        T1[r][cc] = a1;
+        T2[r][cc] = a2;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < D; ++r) {
+      b[r] = bt[r];
+#pragma unroll
+      for (int cc = 0; cc < D; ++cc) A[r][cc] = T1[r][cc];
+#pragma unroll
+      for (int cc = r; cc < D; ++cc) {
+        const int b0 = cc < 4 ? 0 : 4, b1 = cc < 4 ? 4 : D;
+        // the plain term's noise is rounded before the first product joins it
+        F a2 = r < 4 ? Qd[r][cc] : __fadd_rn(Qd[r][cc], 0.f);
+#pragma unroll
+        for (int e = b0; e < b1; ++e) a2 += T2[r][e] * Phi[cc][e];
+        C[r][cc] = a2;
+        C[cc][r] = a2;
+      }
+    }
+    // update with h = e_0 (+ e_4): the latent of the product (and term)
+    const F y = q.y, r0 = q.z;
+    F u[D], g[D];
+#pragma unroll
+    for (int r = 0; r < D; ++r) {
+      u[r] = C[r][0] + (SUM ? C[r][4] : F(0));
+      g[r] = A[0][r] + (SUM ? A[4][r] : F(0));  // h^T A
+    }
+    const F hu = u[0] + (SUM ? u[4] : F(0));
+    const F hb = b[0] + (SUM ? b[4] : F(0));
+    const F Sv = hu + r0 + s2;
+    const F cc = y - hb;
+    bad |= !(Sv > F(0));
+    const F iS = F(1) / Sv;
+    const F ci = cc * iS;
+#pragma unroll
+    for (int r = 0; r < D; ++r) {
+      eta[r] += g[r] * ci;
+#pragma unroll
+      for (int k = 0; k < D; ++k) J[r][k] += g[r] * g[k] * iS;
+    }
+    gam += (double)(cc * ci);
+    ld += glog(Sv);
+    ++n_end;
+#pragma unroll
+    for (int r = 0; r < D; ++r) {
+      const F Kr = u[r] * iS;
+#pragma unroll
+      for (int k = 0; k < D; ++k) A[r][k] -= Kr * g[k];
+      b[r] += Kr * cc;
+#pragma unroll
+      for (int k = 0; k < D; ++k) C[r][k] -= u[r] * u[k] * iS;
+    }
+  }
+  F Cp[ES::NP], Jp[ES::NP];
+#pragma unroll
+  for (int r = 0; r < D; ++r)
+#pragma unroll
+    for (int k = r; k < D; ++k) {
+      Cp[ES::pk(r, k)] = C[r][k];
+      Jp[ES::pk(r, k)] = J[r][k];
+    }
+  store_elem<ES>(ef, n_vch, vc, A, b, Cp, eta, Jp);
+  ed[vc] = gam;
+  ed[(size_t)n_vch + vc] = ld;
+  ed[(size_t)2 * n_vch + vc] = (double)n_end;
+  if (bad) flag_error(err, orow, 7);
+}
+
 template <bool SUM, class ES>
 cudaError_t launch_elem_prod(const DevModel &M, const float *theta, int n_vch, int per_series,
-                             float *ef, double *ed, int *err, const float *, float *, int, float *,
-                             int c_begin, int c_count, float *, int, cudaStream_t st) {
+                             float *ef, double *ed, int *err, const float *, float *, int,
+                             float *sc, int c_begin, int c_count, float *, int, cudaStream_t st) {
   if (n_vch <= 0 || c_count <= 0) return cudaSuccess;
   if (c_begin < 0 || c_begin + c_count > M.n_chunks) return cudaErrorInvalidValue;
-  const int bs = 128;
+  // single warps: a few hundred of them spread over all the SMs
+  const int bs = 32;
   const int64_t nt = (int64_t)(n_vch / M.n_chunks) * c_count;
-  k_elem_prod<SUM, ES><<<(unsigned)((nt + bs - 1) / bs), bs, 0, st>>>(
-      M, theta, n_vch, per_series, ef, ed, err, c_begin, c_count);
+  const unsigned nb = (unsigned)((nt + bs - 1) / bs);
+  if (sc) {
+    k_elem_prod_pre<SUM, ES><<<nb, bs, 0, st>>>(M, theta, n_vch, per_series, ef, ed, err, c_begin,
+                                                c_count, reinterpret_cast<const float4 *>(sc));
+    GPSS_COUNT_LAUNCH();
+  }
+  k_elem_prod<SUM, ES><<<nb, bs, 0, st>>>(M, theta, n_vch, per_series, ef, ed, err, c_begin, c_count,
+                                          sc ? 1 : 0);
   GPSS_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -728,6 +1097,7 @@ OpTable make_prod_ops() {
   o.plain64 = &launch_plain_prod<SUM, double>;
   o.prod_grad = &launch_prod_grad<SUM>;
   o.prod_grad_chunk = &launch_prod_grad_chunk<SUM, ES>;
+  o.prod_scalars = &launch_prod_scalars<SUM>;
   o.tables = &no_tables;
   o.elem = &launch_elem_prod<SUM, ES>;
   o.comb32 = make_combine<ES, float>();
