@@ -40,6 +40,7 @@ namespace gpss {
 constexpr double LOG_2PI = 1.8378770664093454836;
 
 struct DevModel {
+  int n_sm;  // multiprocessors of the device
   int n_series;
   int n_params;
   int n_terms;
@@ -1837,7 +1838,7 @@ __global__ void __launch_bounds__(GRAD_BS, GRAD_MIN_BLOCKS) k_grad(DevModel M, c
 
 // Ordered per-series sums over chunks (deterministic): log-likelihood parts
 // and gradient parts (n_seg records, field-major, stride n_vch), FP64
-// accumulation.
+// accumulation.  One warp per output row and quantity.
 __global__ void k_series_sum(int n_out, int per_series, int n_series, int n_chunks,
                              const int32_t *__restrict__ ch_first,
                              const double *__restrict__ ll_part, int n_vch,
@@ -2184,24 +2185,48 @@ cudaError_t launch_warp_combine(const DevModel &M, const float *ef, int n_vch, v
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  k_warp_scan<S, T><<<(n_vch + 63) / 64, 64, smem, st>>>(ef, n_vch, pre_local, suf_local, wtot,
-                                                         want_info);
+  const int dirs = want_info ? 2 : 1;
+  bool coop = false, coop_fold = false;
+  if constexpr (sizeof(T) == sizeof(float)) {
+    // 16 lanes per combination where one thread each would leave the GPU idle
+    // and take longer alone: states of at least 6 (8 warps of chunks, both
+    // directions: 57 -> 17 us; states of 4, 96 warps: 19 -> 20 us), up to two
+    // blocks per SM (150 warps of states of 6 are 20 us faster, 624 of states
+    // of 7 are 116 us slower)
+    if constexpr (S::D >= 6) {
+      coop = n_w * dirs <= 2 * M.n_sm;
+      if (coop)
+        k_warp_scan_coop<S><<<dim3(n_w, dirs), 32 * COOP, 0, st>>>(ef, n_vch, pre_local,
+                                                                   suf_local, wtot);
+    }
+    // a warp per series and direction until the series alone fill the GPU
+    coop_fold = n_out <= 64 * M.n_sm;
+  }
+  if (!coop)
+    k_warp_scan<S, T><<<(n_vch + 63) / 64, 64, smem, st>>>(ef, n_vch, pre_local, suf_local, wtot,
+                                                           want_info);
   GPSS_COUNT_LAUNCH();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (fold) {
     // few warps per series: sequential fold of the warp totals per series
-    k_warp_fold<S, T><<<(n_out + 63) / 64, 64, 0, st>>>(n_out, per_series, M.n_series,
-                                                        M.n_chunks, M.ch_first, wtot, n_w, wpre,
-                                                        wsuf, want_info);
+    if constexpr (sizeof(T) == sizeof(float)) {
+      if (coop_fold)
+        k_warp_fold_coop<S><<<dim3(n_out, dirs), 32, 0, st>>>(per_series, M.n_series, M.n_chunks,
+                                                              M.ch_first, wtot, n_w, wpre, wsuf);
+    }
+    if (!coop_fold)
+      k_warp_fold<S, T><<<(n_out + 63) / 64, 64, 0, st>>>(n_out, per_series, M.n_series,
+                                                          M.n_chunks, M.ch_first, wtot, n_w, wpre,
+                                                          wsuf, want_info);
     GPSS_COUNT_LAUNCH();
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   } else {
-    e = scan_elems<S, T>(wtot, n_w, wpre, 0, 0, 0, scratch, st);
+    e = scan_elems<S, T>(wtot, n_w, wpre, 0, 0, 0, scratch, M.n_sm, st);
     if (e != cudaSuccess) return e;
     if (want_info) {
-      e = scan_elems<S, T>(wtot, n_w, wsuf, 3, 1, 1, scratch, st);
+      e = scan_elems<S, T>(wtot, n_w, wsuf, 3, 1, 1, scratch, M.n_sm, st);
       if (e != cudaSuccess) return e;
     }
   }
