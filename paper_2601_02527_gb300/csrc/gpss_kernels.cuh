@@ -2194,7 +2194,7 @@ cudaError_t launch_warp_combine(const DevModel &M, const float *ef, int n_vch, v
     // blocks per SM (150 warps of states of 6 are 20 us faster, 624 of states
     // of 7 are 116 us slower)
     if constexpr (S::D >= 6) {
-      coop = n_w * dirs <= 2 * M.n_sm;
+      coop = n_w * dirs <= M.n_sm;
       if (coop)
         k_warp_scan_coop<S><<<dim3(n_w, dirs), 32 * COOP, 0, st>>>(ef, n_vch, pre_local,
                                                                    suf_local, wtot);
@@ -2203,8 +2203,9 @@ cudaError_t launch_warp_combine(const DevModel &M, const float *ef, int n_vch, v
     coop_fold = n_out <= 64 * M.n_sm;
   }
   if (!coop)
-    k_warp_scan<S, T><<<(n_vch + 63) / 64, 64, smem, st>>>(ef, n_vch, pre_local, suf_local, wtot,
-                                                           want_info);
+    // the two directions are independent: blocks of their own
+    k_warp_scan<S, T><<<dim3((n_vch + 63) / 64, dirs), 64, smem, st>>>(ef, n_vch, pre_local,
+                                                                       suf_local, wtot);
   GPSS_COUNT_LAUNCH();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

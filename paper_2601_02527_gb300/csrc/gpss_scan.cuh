@@ -767,7 +767,7 @@ template <class S, class T>
 __global__ void __launch_bounds__(64) k_warp_scan(const float *__restrict__ ef, int n_vch,
                                                   T *__restrict__ pre_local,
                                                   T *__restrict__ suf_local,
-                                                  T *__restrict__ wtot, int want_suffix) {
+                                                  T *__restrict__ wtot) {
   using L = Elem<S>;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   T *sm = reinterpret_cast<T *>(sm_raw);
@@ -778,33 +778,31 @@ __global__ void __launch_bounds__(64) k_warp_scan(const float *__restrict__ ef, 
   if (w >= n_w) return;  // whole warps only (n_vch is a multiple of 32)
   T *bufA = sm + (size_t)(threadIdx.x >> 5) * 2 * 32 * L::NF;
   T *bufB = bufA + 32 * L::NF;
-  for (int dir = 0; dir < (want_suffix ? 2 : 1); ++dir) {
-    for (int f = 0; f < L::NF; ++f) bufA[f * 32 + lane] = T(ef[(size_t)f * n_vch + vc]);
-    __syncwarp();
-    T *src = bufA, *dst = bufB;
-    for (int s = 1; s < 32; s <<= 1) {
-      const bool act = dir == 0 ? lane >= s : lane + s < 32;
-      if (act) {
-        if (dir == 0)
-          combine<S, T>(EViewT<T>{src + lane - s, 32}, EViewT<T>{src + lane, 32},
-                        EViewT<T>{dst + lane, 32});
-        else
-          combine<S, T>(EViewT<T>{src + lane, 32}, EViewT<T>{src + lane + s, 32},
-                        EViewT<T>{dst + lane, 32});
-      } else {
-        copy_elem<S, T>(EViewT<T>{dst + lane, 32}, EViewT<T>{src + lane, 32});
-      }
-      __syncwarp();
-      T *t = src;
-      src = dst;
-      dst = t;
+  const int dir = blockIdx.y;  // 0: prefixes, 1: suffixes
+  for (int f = 0; f < L::NF; ++f) bufA[f * 32 + lane] = T(ef[(size_t)f * n_vch + vc]);
+  __syncwarp();
+  T *src = bufA, *dst = bufB;
+  for (int s = 1; s < 32; s <<= 1) {
+    const bool act = dir == 0 ? lane >= s : lane + s < 32;
+    if (act) {
+      if (dir == 0)
+        combine<S, T>(EViewT<T>{src + lane - s, 32}, EViewT<T>{src + lane, 32},
+                      EViewT<T>{dst + lane, 32});
+      else
+        combine<S, T>(EViewT<T>{src + lane, 32}, EViewT<T>{src + lane + s, 32},
+                      EViewT<T>{dst + lane, 32});
+    } else {
+      copy_elem<S, T>(EViewT<T>{dst + lane, 32}, EViewT<T>{src + lane, 32});
     }
-    T *out = dir == 0 ? pre_local : suf_local;
-    for (int f = 0; f < L::NF; ++f) out[(size_t)f * n_vch + vc] = src[f * 32 + lane];
-    if (dir == 0 && lane == 31)
-      for (int f = 0; f < L::NF; ++f) wtot[(size_t)f * n_w + w] = src[f * 32 + 31];
     __syncwarp();
+    T *t = src;
+    src = dst;
+    dst = t;
   }
+  T *out = dir == 0 ? pre_local : suf_local;
+  for (int f = 0; f < L::NF; ++f) out[(size_t)f * n_vch + vc] = src[f * 32 + lane];
+  if (dir == 0 && lane == 31)
+    for (int f = 0; f < L::NF; ++f) wtot[(size_t)f * n_w + w] = src[f * 32 + 31];
 }
 
 // The same scan with one block per warp of chunks and direction (blockIdx.y)
