@@ -626,7 +626,7 @@ GPSS_HD void elem_event(const Blocks<F> *B, uint8_t tag, F y, F r0, F w, F s2,
 // fields as above plus the number of measurements before that point.  With
 // dcache set, every step's six scalars per term go to the step-scalar cache
 // (for the gradient's forward replay).
-template <class S, bool OD>
+template <class S>
 __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, const float *__restrict__ theta, int n_vch,
                                               int per_series, float *__restrict__ ef,
                                               double *__restrict__ ed, int *__restrict__ err,
@@ -656,10 +656,6 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
   TermC<F> tc[S::NT];
   F s2;
   load_terms<S::NT, F>(theta + (size_t)row * M.n_params, M.kinds, tc, s2);
-  // rows with an overdamped term (and every row of a mixed model) run in the
-  // OD = true launch, the others in the OD = false one (whole warps: a warp's
-  // chunks share one row)
-  if ((any_overdamped<S::NT>(tc) || M.mixed) != OD) return;
   // blocks y > 0: the element of the chunk's segment y - 1 alone (counted from
   // the chunk's end), for the gradient with one thread per segment
   const int seg = (int)blockIdx.y - 1;
@@ -669,81 +665,91 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
   const float4 *tab =
       stage_table<S::NT>(tabs, row, smem_tab + (threadIdx.x >> 5) * (S::NT * TAB_TERM / 4));
   if (seg >= 0 && k_lo <= 0) return;  // nothing precedes the first segment
-  const bool first = seg < 0 && (M.ch_flags[c] & 1);
-  F A[D][D], b[D], C[S::NP], eta[D], J[S::NP];
-  if (first) {
-    init_state<S>(tc, b, C);
-  } else {
+  auto body = [&](auto od_tag) {
+    constexpr bool OD = decltype(od_tag)::value;
+    const bool first = seg < 0 && (M.ch_flags[c] & 1);
+    F A[D][D], b[D], C[S::NP], eta[D], J[S::NP];
+    if (first) {
+      init_state<S>(tc, b, C);
+    } else {
 #pragma unroll
-    for (int i = 0; i < D; ++i) b[i] = F(0);
+      for (int i = 0; i < D; ++i) b[i] = F(0);
 #pragma unroll
-    for (int i = 0; i < S::NP; ++i) C[i] = F(0);
-  }
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
-    eta[i] = F(0);
-#pragma unroll
-    for (int j = 0; j < D; ++j) A[i][j] = (!first && i == j) ? F(1) : F(0);
-  }
-#pragma unroll
-  for (int i = 0; i < S::NP; ++i) J[i] = F(0);
-  double gam = 0.0, ld = 0.0;
-  int n_end = 0;
-  bool bad = false;
-  float4 *dc = dcache_col<S::NT>(M, seg < 0 ? dcache : nullptr, vc);
-  EventReader rd;
-  rd.start(M, c, k_lo, k_hi);
-  // gradient segments end at len - j ck (the first one is the short one);
-  // at each later segment's start the partial element is saved
-  const int f0 = len - ((len - 1) / ck) * ck;
-  int next_ck = pck && seg < 0 ? f0 : len;
-  for (int kk = k_lo; kk < k_hi; ++kk) {
-    if (kk == next_ck) {
-      float *dst = pck + (size_t)((kk - f0) / ck) * (L::NF + 1) * n_vch;
-      store_elem<S>(dst, n_vch, vc, A, b, C, eta, J);
-      dst[(size_t)L::NF * n_vch + vc] = __int_as_float(n_end);
-      next_ck += ck;
+      for (int i = 0; i < S::NP; ++i) C[i] = F(0);
     }
-    F dt;
-    uint8_t tag;
-    float4 q;
-    rd.next(dt, tag, q);
-    Blocks<F> B[S::NT];
-    {
-      constexpr int W = DcW<S::NT>::W;
-      float x[W];
 #pragma unroll
-      for (int t = 0; t < S::NT; ++t) {
-        const Disc<F> d = discretize_tab<OD>(dt, tc[t], tab + t * (TAB_TERM / 4));
-        x[6 * t] = d.f;
-        x[6 * t + 1] = d.fp;
-        x[6 * t + 2] = d.F1;
-        x[6 * t + 3] = d.Iff;
-        x[6 * t + 4] = d.Ipp;
-        x[6 * t + 5] = d.IFF;
-        B[t] = make_blocks(d, tc[t]);
-      }
+    for (int i = 0; i < D; ++i) {
+      eta[i] = F(0);
 #pragma unroll
-      for (int i = 6 * S::NT; i < W; ++i) x[i] = 0.f;
-      if (dc) {
-        float4 *r = dc + (size_t)kk * (32 * DcW<S::NT>::G);
-#pragma unroll
-        for (int v = 0; v < DcW<S::NT>::G; ++v)
-          r[32 * v] = make_float4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
-      }
+      for (int j = 0; j < D; ++j) A[i][j] = (!first && i == j) ? F(1) : F(0);
     }
-    elem_event<S, F, OD>(B, tag, q.x, q.y, q.z, s2, A, b, C, eta, J, gam, ld, n_end, bad);
-  }
-  if (seg >= 0) {
-    store_elem<S>(segel + (size_t)seg * L::NF * n_vch, n_vch, vc, A, b, C, eta, J);
+#pragma unroll
+    for (int i = 0; i < S::NP; ++i) J[i] = F(0);
+    double gam = 0.0, ld = 0.0;
+    int n_end = 0;
+    bool bad = false;
+    float4 *dc = dcache_col<S::NT>(M, seg < 0 ? dcache : nullptr, vc);
+    EventReader rd;
+    rd.start(M, c, k_lo, k_hi);
+    // gradient segments end at len - j ck (the first one is the short one);
+    // at each later segment's start the partial element is saved
+    const int f0 = len - ((len - 1) / ck) * ck;
+    int next_ck = pck && seg < 0 ? f0 : len;
+    for (int kk = k_lo; kk < k_hi; ++kk) {
+      if (kk == next_ck) {
+        float *dst = pck + (size_t)((kk - f0) / ck) * (L::NF + 1) * n_vch;
+        store_elem<S>(dst, n_vch, vc, A, b, C, eta, J);
+        dst[(size_t)L::NF * n_vch + vc] = __int_as_float(n_end);
+        next_ck += ck;
+      }
+      F dt;
+      uint8_t tag;
+      float4 q;
+      rd.next(dt, tag, q);
+      Blocks<F> B[S::NT];
+      {
+        constexpr int W = DcW<S::NT>::W;
+        float x[W];
+#pragma unroll
+        for (int t = 0; t < S::NT; ++t) {
+          const Disc<F> d = discretize_tab<OD>(dt, tc[t], tab + t * (TAB_TERM / 4));
+          x[6 * t] = d.f;
+          x[6 * t + 1] = d.fp;
+          x[6 * t + 2] = d.F1;
+          x[6 * t + 3] = d.Iff;
+          x[6 * t + 4] = d.Ipp;
+          x[6 * t + 5] = d.IFF;
+          B[t] = make_blocks(d, tc[t]);
+        }
+#pragma unroll
+        for (int i = 6 * S::NT; i < W; ++i) x[i] = 0.f;
+        if (dc) {
+          float4 *r = dc + (size_t)kk * (32 * DcW<S::NT>::G);
+#pragma unroll
+          for (int v = 0; v < DcW<S::NT>::G; ++v)
+            r[32 * v] = make_float4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
+        }
+      }
+      elem_event<S, F, OD>(B, tag, q.x, q.y, q.z, s2, A, b, C, eta, J, gam, ld, n_end, bad);
+    }
+    if (seg >= 0) {
+      store_elem<S>(segel + (size_t)seg * L::NF * n_vch, n_vch, vc, A, b, C, eta, J);
+      if (bad) flag_error(err, orow, 7);
+      return;
+    }
+    store_elem<S>(ef, n_vch, vc, A, b, C, eta, J);
+    ed[vc] = gam;
+    ed[(size_t)n_vch + vc] = ld;
+    ed[(size_t)2 * n_vch + vc] = (double)n_end;
     if (bad) flag_error(err, orow, 7);
-    return;
-  }
-  store_elem<S>(ef, n_vch, vc, A, b, C, eta, J);
-  ed[vc] = gam;
-  ed[(size_t)n_vch + vc] = ld;
-  ed[(size_t)2 * n_vch + vc] = (double)n_end;
-  if (bad) flag_error(err, orow, 7);
+};
+  // rows with an overdamped term, and every row of a mixed model, take the
+  // general body, the others the lean one (whole warps: a warp's chunks share
+  // one row)
+  if (any_overdamped<S::NT>(tc) || M.mixed)
+    body(OdTag<true>{});
+  else
+    body(OdTag<false>{});
 }
 
 // ---------------------------------------------------------------------------
@@ -2116,16 +2122,11 @@ cudaError_t launch_elem(const DevModel &M, const float *theta, int n_vch, int pe
   if (pck && (ck < 2 || ck > 64 || (ck & 1))) return cudaErrorInvalidValue;
   const int bs = ELEM_BS;
   const size_t smem = (size_t)(bs / 32) * S::NT * TAB_TERM * sizeof(float);
-  // two launches: rows without an overdamped term (the lean body), then rows
-  // with one; each skips the other's rows
   const int64_t nt = (int64_t)(n_vch / M.n_chunks) * c_count;
   // every segment's own element but the first one's beside the chunks'
   const dim3 nb((unsigned)((nt + bs - 1) / bs), segel ? n_seg : 1);
-  k_elem<S, false><<<nb, bs, smem, st>>>(M, theta, n_vch, per_series, ef, ed, err, tabs, pck,
-                                         pck ? ck : 1, dcache, c_begin, c_count, segel);
-  GPSS_COUNT_LAUNCH();
-  k_elem<S, true><<<nb, bs, smem, st>>>(M, theta, n_vch, per_series, ef, ed, err, tabs, pck,
-                                        pck ? ck : 1, dcache, c_begin, c_count, segel);
+  k_elem<S><<<nb, bs, smem, st>>>(M, theta, n_vch, per_series, ef, ed, err, tabs, pck,
+                                  pck ? ck : 1, dcache, c_begin, c_count, segel);
   GPSS_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -2190,9 +2191,9 @@ cudaError_t launch_warp_combine(const DevModel &M, const float *ef, int n_vch, v
   if constexpr (sizeof(T) == sizeof(float)) {
     // 16 lanes per combination where one thread each would leave the GPU idle
     // and take longer alone: states of at least 6 (8 warps of chunks, both
-    // directions: 57 -> 17 us; states of 4, 96 warps: 19 -> 20 us), up to two
-    // blocks per SM (150 warps of states of 6 are 20 us faster, 624 of states
-    // of 7 are 116 us slower)
+    // directions: 57 -> 17 us; states of 4, 96 warps: 19 -> 20 us), up to one
+    // block per SM (150 warps of states of 6, 300 blocks: 40 us against 33 with
+    // one thread; 624 of states of 7: 236 against 101)
     if constexpr (S::D >= 6) {
       coop = n_w * dirs <= M.n_sm;
       if (coop)

@@ -757,6 +757,12 @@ cudaError_t scan_elems(const T *src, int n, T *dst, int mode, int rev_index, int
 // than chunks -- are then scanned by scan_elems (or folded per series), and
 // k_join combines the two levels per chunk.  T is the arithmetic of every
 // combination (the chunk elements themselves are FP32).
+//
+// Bound by the instruction caches and the serial chain of a combination where
+// warps are few, by instruction issue where they are many.  The directions
+// are independent blocks (blockIdx.y) that share one copy of the combination's
+// code: 357 warps, states of 5: 34 -> 21 us; 2430 warps, states of 6: 149 ->
+// 132 us against one after the other, each with its own copy.
 // ---------------------------------------------------------------------------
 template <class S, class T>
 constexpr size_t warp_scan_smem_bytes(int warps) {
@@ -785,12 +791,9 @@ __global__ void __launch_bounds__(64) k_warp_scan(const float *__restrict__ ef, 
   for (int s = 1; s < 32; s <<= 1) {
     const bool act = dir == 0 ? lane >= s : lane + s < 32;
     if (act) {
-      if (dir == 0)
-        combine<S, T>(EViewT<T>{src + lane - s, 32}, EViewT<T>{src + lane, 32},
-                      EViewT<T>{dst + lane, 32});
-      else
-        combine<S, T>(EViewT<T>{src + lane, 32}, EViewT<T>{src + lane + s, 32},
-                      EViewT<T>{dst + lane, 32});
+      // one copy of the combination's code serves both directions
+      T *early = src + (dir == 0 ? lane - s : lane), *late = src + (dir == 0 ? lane : lane + s);
+      combine<S, T>(EViewT<T>{early, 32}, EViewT<T>{late, 32}, EViewT<T>{dst + lane, 32});
     } else {
       copy_elem<S, T>(EViewT<T>{dst + lane, 32}, EViewT<T>{src + lane, 32});
     }
