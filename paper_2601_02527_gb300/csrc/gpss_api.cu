@@ -14,6 +14,7 @@
 
 #include "gpss.h"
 #include "gpss_kernels.cuh"
+#include "gpss_plan.h"
 
 namespace gpss {
 OpTable ops_1_1_0();
@@ -912,33 +913,6 @@ struct ElemSlices {
   const cudaEvent_t *ready;
 };
 
-// Segments of ck events per chunk that the gradient walks in parallel, one
-// thread each (1: one thread per chunk walks them in turn).  A thread takes
-// the serial time of its events, so too few chunks leave the GPU idle;
-// parallel segments cost each segment's own element beside the chunk's and a
-// boundary adjoint per segment.  The line lies where both take the same time:
-// 6 warps of chunks per SM, 12 for states of at most 4 (cheaper elements).
-// One call, parallel against in turn, 152 SMs: two SHO terms 911 warps 1254
-// us against 1367, 1215 warps 1534 against 1418; SHO + Matern-3/2 with three
-// slots 624 warps 1674 against 1935, 936 warps 2136 each; instants 1205
-// warps 1009 against 1152, 1649 warps 1279 against 1300.  The adjoint at a
-// segment's end differs from the walked one in rounding; exposure gradients
-// and predictions, differences of nearly equal terms, would show it at 3e-5
-// of their size and keep the walk in turn.
-int grad_segments(const gp_ss_model *m, int n_vch, int ck) {
-  constexpr int kMaxSegments = 1024;  // k_seg_info carries the adjoints back through them in turn
-  constexpr size_t kMaxReplay = (size_t)2 << 30;  // bytes of the replay buffers
-  // shorter segments would put a boundary adjoint's rounding every few events
-  if (m->product || ck < 32) return 1;
-  const OpTable &o = m->ops;
-  const int n_seg = (m->max_chunk + ck - 1) / ck;
-  const int per_sm = o.D <= 4 ? 12 : 6;
-  if (n_vch / 32 > per_sm * m->n_sm || n_seg < 2 || n_seg > kMaxSegments) return 1;
-  const size_t replay =
-      (size_t)n_seg * ck * (4 * ((o.D + o.NP + 3) / 4)) * n_vch * sizeof(float);
-  return replay <= kMaxReplay ? n_seg : 1;
-}
-
 // Test times of a prediction, sorted and uploaded while the GPU runs the
 // element pass and the combination, which do not need them: enqueue calls
 // upload just before the gradient walk.  The host block and its device copy
@@ -1095,8 +1069,11 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
     // every recomputation segment but a chunk's first
     const int ck = m->ckpt_interval;
     const int n_pck = std::max((m->max_chunk - 1) / ck, 1);
-    int n_seg = grad && tree && !dexp && !pred ? grad_segments(m, n_vch, ck) : 1;
-    const size_t replay = (size_t)ck * (4 * ((SD + 3) / 4)) * n_vch * sizeof(float);
+    int n_seg = grad && tree && !dexp && !pred
+                    ? gpss::grad_segments({m->product, m->comb_prec, o.D, o.NP, m->max_chunk, ck,
+                                           n_vch, m->n_sm})
+                    : 1;
+    const size_t replay = gpss::replay_bytes(ck, o.D, o.NP, n_vch, 1);
     if (!grab((void **)&ef, (size_t)o.NF * n_vch * sizeof(float)) ||
         !grab((void **)&ed, (size_t)o.ND * n_vch * sizeof(double)) ||
         !grab((void **)&tabs, (size_t)n_sets * o.NT * gpss::TAB_TERM * sizeof(float)) ||

@@ -1,0 +1,52 @@
+// Rules by which a call's work is laid out that need no device: plain C++, so
+// that the CPU tests compile and check them as they are.
+#pragma once
+
+#include <cstddef>
+
+namespace gpss {
+
+// What the choice between parallel and serial gradient segments looks at.
+struct SegmentCase {
+  bool product;   // product kernel: forward-mode tangents, no segments
+  int comb_prec;  // arithmetic of the cross-chunk combination: 32 or 64
+  int D, NP;      // state dimension and its packed covariance
+  int max_chunk;  // events of the longest chunk
+  int ck;         // events per segment
+  int n_vch;      // chunks of the call (all parameter sets)
+  int n_sm;       // multiprocessors
+};
+
+// Bytes of the replay buffers of n_seg segments per chunk.
+inline size_t replay_bytes(int ck, int D, int NP, int n_vch, int n_seg) {
+  return (size_t)n_seg * ck * (4 * ((D + NP + 3) / 4)) * n_vch * sizeof(float);
+}
+
+// Segments of ck events per chunk that the gradient walks in parallel, one
+// thread each (1: one thread per chunk walks them in turn).  A thread takes
+// the serial time of its events, so too few chunks leave the GPU idle;
+// parallel segments cost each segment's own element beside the chunk's and a
+// boundary adjoint per segment.  The line lies where both take the same time:
+// 6 warps of chunks per SM, 12 for states of at most 4 (cheaper elements).
+// One call, parallel against in turn, 152 SMs: two SHO terms 911 warps 1254
+// us against 1367, 1215 warps 1534 against 1418; SHO + Matern-3/2 with three
+// slots 624 warps 1674 against 1935, 936 warps 2136 each; instants 1205
+// warps 1009 against 1152, 1649 warps 1279 against 1300.  The adjoint at a
+// segment's end differs from the walked one in rounding; exposure gradients
+// and predictions, differences of nearly equal terms, would show it at 3e-5
+// of their size and keep the walk in turn.  The segments' elements and the
+// information carried back through them are FP32: a model whose combination
+// runs in FP64 starts the walk in turn from the FP64 adjoint at the chunk's
+// end and keeps it.
+inline int grad_segments(const SegmentCase &c) {
+  constexpr int kMaxSegments = 1024;  // k_seg_info carries the adjoints back through them in turn
+  constexpr size_t kMaxReplay = (size_t)2 << 30;  // bytes of the replay buffers
+  // shorter segments would put a boundary adjoint's rounding every few events
+  if (c.product || c.comb_prec != 32 || c.ck < 32) return 1;
+  const int n_seg = (c.max_chunk + c.ck - 1) / c.ck;
+  const int per_sm = c.D <= 4 ? 12 : 6;
+  if (c.n_vch / 32 > per_sm * c.n_sm || n_seg < 2 || n_seg > kMaxSegments) return 1;
+  return replay_bytes(c.ck, c.D, c.NP, c.n_vch, n_seg) <= kMaxReplay ? n_seg : 1;
+}
+
+}  // namespace gpss

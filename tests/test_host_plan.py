@@ -1,0 +1,43 @@
+"""The rules by which a call is laid out (csrc/gpss_plan.h), compiled for the
+host as they are."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "hostmath")
+CSRC = os.path.join(os.path.dirname(os.path.dirname(HERE)), "paper_2601_02527_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def plan():
+    src = os.path.join(HERE, "gpss_plan_harness.cpp")
+    out = os.path.join(HERE, "_build", "libgpss_plan.so")
+    os.makedirs(os.path.dirname(out), exist_ok=True)
+    tmp = out + f".tmp{os.getpid()}"
+    subprocess.check_call(["g++", "-O1", "-Wall", "-Werror", "-std=c++17", "-fPIC", "-shared",
+                           "-I", CSRC, src, "-o", tmp])
+    os.replace(tmp, out)
+    return ctypes.CDLL(out)
+
+
+# product, combination precision, D, longest chunk, ck, chunks, SMs -> segments
+@pytest.mark.parametrize("case,want", [
+    ((0, 32, 6, 256, 32, 320, 152), 8),
+    ((0, 32, 6, 33, 32, 320, 152), 2),
+    ((0, 32, 6, 32, 32, 320, 152), 1),             # one segment is the chunk
+    ((0, 64, 6, 256, 32, 320, 152), 1),            # FP64 adjoints at chunk ends: walked on
+    ((0, 64, 3, 256, 64, 320, 152), 1),
+    ((0, 32, 6, 256, 16, 320, 152), 1),            # short segments
+    ((1, 32, 4, 256, 32, 320, 152), 1),            # product kernels have none
+    ((0, 32, 6, 256, 32, 32 * 6 * 152, 152), 8),   # the line, and past it
+    ((0, 32, 6, 256, 32, 32 * (6 * 152 + 1), 152), 1),
+    ((0, 32, 4, 256, 32, 32 * 12 * 152, 152), 8),
+    ((0, 32, 4, 256, 32, 32 * (12 * 152 + 1), 152), 1),
+    ((0, 32, 6, 32 * 1024, 32, 32, 152), 1024),
+    ((0, 32, 6, 32 * 1024 + 1, 32, 32, 152), 1),
+    ((0, 32, 7, 1024, 32, 29184, 152), 1),         # past 2 GiB of replay
+])
+def test_segments_of_a_gradient(plan, case, want):
+    assert plan.ph_grad_segments(*case) == want
