@@ -1050,18 +1050,26 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
   // (default), or the sequential fold with one thread per series
   bool tree = m->combine != 1;
   std::vector<void *> bufs;
-  auto grab = [&](void **p, size_t bytes) -> bool {
-    if (scratch_alloc(m, p, std::max<size_t>(bytes, 16), st) != cudaSuccess) {
-      *p = nullptr;
+  auto take = [&](void **p, size_t bytes) {
+    if (scratch_alloc(m, p, bytes, st) != cudaSuccess) {
+      cudaGetLastError();
       return false;
     }
     bufs.push_back(*p);
     return true;
   };
+  auto give = [&] {
+    cudaFreeAsync(bufs.back(), st);
+    bufs.pop_back();
+  };
   float *ef = nullptr, *adj = nullptr, *ckpt = nullptr, *gpart = nullptr, *tabs = nullptr;
   float *segel = nullptr, *seg_info = nullptr, *seg_adj = nullptr, *rbuf = nullptr;
-  int n_gpart = 1;
+  float *dcache = nullptr, *ptan = nullptr, *gdt = nullptr, *gwe = nullptr;
+  float2 *cond = nullptr;
   void *state_end = nullptr, *info = nullptr, *scratch = nullptr;
+  // warp-level combination buffers
+  void *pre_local = nullptr, *suf_local = nullptr, *wtot = nullptr, *wpre = nullptr,
+       *wsuf = nullptr;
   double *ed = nullptr, *ll_part = nullptr;
   gp_ss_status res = GP_SS_OK;
   do {
@@ -1073,54 +1081,87 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
                     ? gpss::grad_segments({m->product, m->comb_prec, o.D, o.NP, m->max_chunk, ck,
                                            n_vch, m->n_sm})
                     : 1;
-    const size_t replay = gpss::replay_bytes(ck, o.D, o.NP, n_vch, 1);
-    if (!grab((void **)&ef, (size_t)o.NF * n_vch * sizeof(float)) ||
-        !grab((void **)&ed, (size_t)o.ND * n_vch * sizeof(double)) ||
-        !grab((void **)&tabs, (size_t)n_sets * o.NT * gpss::TAB_TERM * sizeof(float)) ||
-        (grad && !m->product &&
-         !grab((void **)&ckpt, (size_t)n_pck * (o.NF + 1) * n_vch * sizeof(float)))) {
+    const size_t nv = (size_t)n_vch, n_w = nv / 32, rows = nv / m->n_chunks;
+    const size_t exp_ev = (size_t)(per_series ? 1 : n_sets) * m->n_events;
+    const size_t part = m->n_params * nv * sizeof(float);
+    std::vector<gpss::Buffer> needed, fast, plain;
+    auto put = [](std::vector<gpss::Buffer> &list, auto &p, size_t bytes) {
+      list.push_back({(void **)&p, bytes});
+    };
+    put(needed, ef, o.NF * nv * sizeof(float));
+    put(needed, ed, o.ND * nv * sizeof(double));
+    put(needed, tabs, (size_t)n_sets * o.NT * gpss::TAB_TERM * sizeof(float));
+    if (grad || tree) put(needed, state_end, SD * nv * eb);
+    if (tree) {
+      put(needed, ll_part, nv * sizeof(double));
+      put(needed, pre_local, o.NF * nv * eb);
+      put(needed, wtot, o.NF * n_w * eb);
+      put(needed, wpre, o.NF * n_w * eb);
+      put(needed, scratch, cb.warp_scratch(n_vch) * eb);
+      if (grad) {
+        put(needed, info, SD * nv * eb);
+        put(needed, suf_local, o.NF * nv * eb);
+        put(needed, wsuf, o.NF * n_w * eb);
+      }
+    }
+    if (grad) put(needed, adj, SD * nv * sizeof(float));
+    if (dexp) {
+      put(needed, gdt, exp_ev * sizeof(float));
+      put(needed, gwe, exp_ev * sizeof(float));
+    }
+    if (cond_out) put(needed, cond, exp_ev * sizeof(float2));
+    if (m->product) {
+      if (grad) put(needed, gpart, part);
+      // the oscillators' scalars of every step (the gradient's with their
+      // tangents); without them every thread forms its own step by step
+      const size_t bytes = rows * (size_t)m->dcache_steps * (o.D / 2) * sizeof(float4);
+      if (m->step_cache == 0 && m->max_chunk <= 65535 * gpss::PROD_STEPS &&
+          bytes * (grad ? 3 : 1) <= kDcacheMax) {
+        put(fast, dcache, bytes);
+        if (grad) put(fast, ptan, 2 * bytes);
+      }
+    } else if (grad) {
+      put(needed, ckpt, n_pck * (o.NF + 1) * nv * sizeof(float));
+      // the element pass keeps every step's scalars for the gradient's replay
+      // while that takes at most kDcacheMax bytes (else the replay recomputes them)
+      const size_t bytes =
+          rows * (size_t)m->dcache_steps * (4 * ((6 * o.NT + 3) / 4)) * sizeof(float);
+      if (m->step_cache == 0 && bytes <= kDcacheMax) put(needed, dcache, bytes);
+      put(plain, rbuf, gpss::replay_bytes(ck, o.D, o.NP, n_vch, 1));
+      put(plain, gpart, part);
+      if (n_seg > 1) {
+        const size_t rec = (n_seg - 1) * nv * sizeof(float);
+        // the largest first: where a later one fails, the plain way's replay
+        // fits into what this one gives back
+        put(fast, rbuf, gpss::replay_bytes(ck, o.D, o.NP, n_vch, n_seg));
+        put(fast, segel, rec * o.NF);
+        put(fast, seg_info, rec * SD);
+        put(fast, seg_adj, rec * SD);
+        put(fast, gpart, n_seg * part);
+      }
+    }
+    // a capture records allocations without making them, and a graph's come in
+    // larger pieces: the fast way's are recorded only if the device has twice
+    // the call's memory now (free, or kept by graphs that ended)
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (!fast.empty() && cudaStreamIsCapturing(st, &cs) == cudaSuccess &&
+        cs != cudaStreamCaptureStatusNone) {
+      size_t avail = 0, total = 0;
+      uint64_t kept = 0, used = 0;
+      if (cudaMemGetInfo(&avail, &total) != cudaSuccess ||
+          cudaDeviceGetGraphMemAttribute(m->device, cudaGraphMemAttrReservedMemCurrent, &kept) !=
+              cudaSuccess ||
+          cudaDeviceGetGraphMemAttribute(m->device, cudaGraphMemAttrUsedMemCurrent, &used) !=
+              cudaSuccess ||
+          2 * (gpss::total_bytes(needed) + gpss::total_bytes(fast)) > avail + (kept - used))
+        fast.clear();
+    }
+    const gpss::Scratch way = gpss::take_scratch(needed, fast, plain, take, give);
+    if (way == gpss::Scratch::none) {
       res = GP_SS_ENOMEM;
       break;
     }
-    // the element pass keeps every step's scalars for the gradient's replay
-    // while that takes at most kDcacheMax bytes (else the replay recomputes them)
-    float *dcache = nullptr;
-    if (grad && !m->product) {
-      const size_t dbytes = (size_t)(n_vch / m->n_chunks) * (size_t)m->dcache_steps *
-                            (4 * ((6 * o.NT + 3) / 4)) * sizeof(float);
-      if (m->step_cache == 0 && dbytes <= kDcacheMax && !grab((void **)&dcache, dbytes)) {
-        res = GP_SS_ENOMEM;
-        break;
-      }
-    }
-    if (n_seg > 1) {
-      // without the memory for parallel segments they are walked in turn
-      const size_t before = bufs.size(), rec = (size_t)(n_seg - 1) * n_vch * sizeof(float);
-      if (!grab((void **)&segel, rec * o.NF) || !grab((void **)&seg_info, rec * SD) ||
-          !grab((void **)&seg_adj, rec * SD) || !grab((void **)&rbuf, replay * n_seg)) {
-        while (bufs.size() > before) {
-          cudaFreeAsync(bufs.back(), st);
-          bufs.pop_back();
-        }
-        cudaGetLastError();
-        segel = seg_info = seg_adj = rbuf = nullptr;
-        n_seg = 1;
-      }
-    }
-    // product models: the oscillators' scalars of every step (the gradient's
-    // with their tangents), within the same bound and where the memory is there
-    float *ptan = nullptr;
-    if (m->product && m->step_cache == 0 && m->max_chunk <= 65535 * gpss::PROD_STEPS) {
-      const size_t bytes =
-          (size_t)(n_vch / m->n_chunks) * (size_t)m->dcache_steps * (o.D / 2) * sizeof(float4);
-      if (bytes * (grad ? 3 : 1) <= kDcacheMax && grab((void **)&dcache, bytes) && grad &&
-          !grab((void **)&ptan, 2 * bytes)) {
-        cudaFreeAsync(dcache, st);
-        bufs.pop_back();
-        dcache = nullptr;
-      }
-      cudaGetLastError();
-    }
+    if (way == gpss::Scratch::plain) n_seg = 1;
     {
       PhaseTimer pt(m, st, 0);
       if (m->product && dcache &&
@@ -1147,28 +1188,6 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
       }
       if (res) break;
     }
-    if ((grad || tree) && !grab(&state_end, (size_t)SD * n_vch * eb)) {
-      res = GP_SS_ENOMEM;
-      break;
-    }
-    if (grad && !grab((void **)&adj, (size_t)SD * n_vch * sizeof(float))) {
-      res = GP_SS_ENOMEM;
-      break;
-    }
-    // warp-level combination buffers
-    void *pre_local = nullptr, *suf_local = nullptr, *wtot = nullptr, *wpre = nullptr,
-         *wsuf = nullptr;
-    const int n_w = n_vch / 32;
-    if (tree && (!grab((void **)&ll_part, (size_t)n_vch * sizeof(double)) ||
-                 !grab(&pre_local, (size_t)o.NF * n_vch * eb) ||
-                 !grab(&wtot, (size_t)o.NF * n_w * eb) || !grab(&wpre, (size_t)o.NF * n_w * eb) ||
-                 !grab(&scratch, cb.warp_scratch(n_vch) * eb) ||
-                 (grad && (!grab(&info, (size_t)SD * n_vch * eb) ||
-                           !grab(&suf_local, (size_t)o.NF * n_vch * eb) ||
-                           !grab(&wsuf, (size_t)o.NF * n_w * eb))))) {
-      res = GP_SS_ENOMEM;
-      break;
-    }
     {
       PhaseTimer pt(m, st, 1);
       cudaError_t e;
@@ -1190,20 +1209,7 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
       }
     }
     if (grad) {
-      float *gdt = nullptr, *gwe = nullptr;
-      float2 *cond = nullptr;
       const int exp_rows = per_series ? 1 : n_sets;
-      if ((dexp && (!grab((void **)&gdt, (size_t)exp_rows * m->n_events * sizeof(float)) ||
-                    !grab((void **)&gwe, (size_t)exp_rows * m->n_events * sizeof(float)))) ||
-          (cond_out && !grab((void **)&cond, (size_t)exp_rows * m->n_events * sizeof(float2)))) {
-        res = GP_SS_ENOMEM;
-        break;
-      }
-      if ((!m->product && !rbuf && !grab((void **)&rbuf, replay)) ||
-          !grab((void **)&gpart, (size_t)n_seg * m->n_params * n_vch * sizeof(float))) {
-        res = GP_SS_ENOMEM;
-        break;
-      }
       PhaseTimer pt(m, st, 2);
       if (m->product) {
         // chunked forward-mode tangents against the boundary adjoints
@@ -1214,7 +1220,6 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
       } else {
         gpss::PredPlan pp;
         if (pred && (res = pred->upload(&pp, st))) break;
-        n_gpart = n_seg;
         if ((n_seg > 1 && o.seg_adjoint(dm, n_vch, state_end, info, eb == 8 ? 1 : 0, ckpt, segel,
                                         seg_info, seg_adj, ck, n_seg, st)) ||
             o.grad(dm, theta, n_vch, per_series, state_end, eb == 8 ? 1 : 0, adj, ckpt, gpart,
@@ -1252,7 +1257,7 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
       const int64_t sums = (int64_t)n_out * ((tree ? 1 : 0) + (grad ? m->n_params : 0));
       gpss::k_series_sum<<<(unsigned)((sums * 32 + 127) / 128), 128, 0, st>>>(
           n_out, per_series, m->n_series, m->n_chunks, m->d_ch_first, tree ? ll_part : nullptr,
-          n_vch, grad ? gpart : nullptr, n_gpart, m->n_params, ll, grad);
+          n_vch, grad ? gpart : nullptr, n_seg, m->n_params, ll, grad);
       GPSS_COUNT_LAUNCH();
       if (cudaGetLastError() != cudaSuccess) res = GP_SS_ECUDA;
     }

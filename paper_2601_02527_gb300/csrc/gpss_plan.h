@@ -2,7 +2,9 @@
 // that the CPU tests compile and check them as they are.
 #pragma once
 
+#include <algorithm>
 #include <cstddef>
+#include <vector>
 
 namespace gpss {
 
@@ -47,6 +49,45 @@ inline int grad_segments(const SegmentCase &c) {
   const int per_sm = c.D <= 4 ? 12 : 6;
   if (c.n_vch / 32 > per_sm * c.n_sm || n_seg < 2 || n_seg > kMaxSegments) return 1;
   return replay_bytes(c.ck, c.D, c.NP, c.n_vch, n_seg) <= kMaxReplay ? n_seg : 1;
+}
+
+// Scratch buffers of one call: *p receives the address.
+struct Buffer {
+  void **p;
+  size_t bytes;
+};
+
+inline size_t total_bytes(const std::vector<Buffer> &list) {
+  size_t n = 0;
+  for (const Buffer &b : list) n += b.bytes;
+  return n;
+}
+
+// Takes every buffer of the list; when one cannot be had, gives back those
+// before it and leaves all null.  take(p, bytes) says whether it succeeded,
+// give() returns the buffer taken last.
+template <class Take, class Give>
+bool take_all(const std::vector<Buffer> &list, Take take, Give give) {
+  for (size_t i = 0; i < list.size(); ++i) {
+    if (take(list[i].p, std::max<size_t>(list[i].bytes, 16))) continue;
+    for (; i > 0; --i) give();
+    for (const Buffer &b : list) *b.p = nullptr;
+    return false;
+  }
+  return true;
+}
+
+enum class Scratch { none, plain, fast };
+
+// A call's scratch: what both of its ways need, then the buffers of the fast
+// way or, where they cannot be had, of the plain one.  The fast way's are
+// taken last, so that a call is refused only where the plain way does not fit.
+template <class Take, class Give>
+Scratch take_scratch(const std::vector<Buffer> &needed, const std::vector<Buffer> &fast,
+                     const std::vector<Buffer> &plain, Take take, Give give) {
+  if (!take_all(needed, take, give)) return Scratch::none;
+  if (!fast.empty() && take_all(fast, take, give)) return Scratch::fast;
+  return take_all(plain, take, give) ? Scratch::plain : Scratch::none;
 }
 
 }  // namespace gpss

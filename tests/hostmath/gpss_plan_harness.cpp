@@ -11,4 +11,30 @@ int ph_grad_segments(int product, int comb_prec, int D, int max_chunk, int ck, i
   return grad_segments({product != 0, comb_prec, D, D * (D + 1) / 2, max_chunk, ck, n_vch, n_sm});
 }
 
+// take_scratch against an allocator of `limit` bytes.  n[3], bytes: the lists
+// (needed, fast, plain) one after the other; held: bytes taken in the end;
+// got[i]: buffer i is in hand.  Returns 0 none, 1 plain, 2 fast.
+int ph_take_scratch(size_t limit, const int *n, const size_t *bytes, size_t *held, int *got) {
+  std::vector<void *> addr(n[0] + n[1] + n[2], (void *)8);
+  std::vector<Buffer> list[3];
+  for (int l = 0, i = 0; l < 3; ++l)
+    for (int k = 0; k < n[l]; ++k, ++i) list[l].push_back({&addr[i], bytes[i]});
+  std::vector<size_t> taken;
+  *held = 0;
+  auto take = [&](void **p, size_t b) {
+    *p = (void *)8;  // a failed allocation may leave anything
+    if (*held + b > limit) return false;
+    *held += b;
+    taken.push_back(b);
+    return true;
+  };
+  auto give = [&] {
+    *held -= taken.back();
+    taken.pop_back();
+  };
+  const Scratch way = take_scratch(list[0], list[1], list[2], take, give);
+  for (size_t i = 0; i < addr.size(); ++i) got[i] = addr[i] != nullptr;
+  return way == Scratch::none ? 0 : way == Scratch::plain ? 1 : 2;
+}
+
 }  // extern "C"

@@ -41,3 +41,29 @@ def plan():
 ])
 def test_segments_of_a_gradient(plan, case, want):
     assert plan.ph_grad_segments(*case) == want
+
+
+# bytes of the buffers: needed, of the fast way, of the plain way
+@pytest.mark.parametrize("needed,fast,plain", [
+    ([100, 40, 16], [800, 70, 30], [100, 16]),     # segments of a gradient
+    ([100, 40, 16], [300, 600], []),               # a product model's scalars
+    ([100, 40, 16], [], [50]),
+    ([100], [64], [64]),
+])
+def test_scratch_is_refused_only_where_the_plain_way_does_not_fit(plan, needed, fast, plain):
+    lists = [needed, fast, plain]
+    n = (ctypes.c_int * 3)(*[len(x) for x in lists])
+    flat = sum(lists, [])
+    size = (ctypes.c_size_t * len(flat))(*flat)
+    for limit in range(sum(needed) + sum(fast) + sum(plain) + 2):
+        held, got = ctypes.c_size_t(), (ctypes.c_int * len(flat))()
+        way = plan.ph_take_scratch(ctypes.c_size_t(limit), n, size, ctypes.byref(held), got)
+        with_fast, with_plain = sum(needed) + sum(fast), sum(needed) + sum(plain)
+        want = 2 if fast and with_fast <= limit else int(with_plain <= limit)
+        assert way == want, (limit, way)
+        if way == 2:
+            assert held.value == with_fast and all(got[:len(needed) + len(fast)])
+        elif way == 1:
+            assert held.value == with_plain
+            assert list(got)[:len(flat) - len(plain)] == [1] * len(needed) + [0] * len(fast)
+            assert all(list(got)[len(flat) - len(plain):])
