@@ -1706,15 +1706,8 @@ gp_ss_status gp_ss_loglik_grad_host(const gp_ss_model *m, const float *theta_hos
   // A re-sent event stream goes up in series groups on a second stream, and
   // each group's element pass starts as soon as its events are in (the copy
   // of the rest overlaps it).  The copy stream first waits for earlier work
-  // on st, which may still read the device copy.  A group's element pass takes
-  // at least its longest chunk's serial time however few chunks it has, so a
-  // group is given at least one block of chunks per SM, and there are at most
-  // four groups (90112 chunks of two terms: element phase with the upload
-  // 1.84 ms with four, 1.90 ms with two; 11424 chunks: the whole call 1.75 ms
-  // with four, 1.17 ms with one).
-  constexpr int kGroups = 4;
-  const int n_groups =
-      std::max(1, std::min(kGroups, m->n_chunks / std::max(1, m->n_sm * gpss::ELEM_BS)));
+  // on st, which may still read the device copy.
+  constexpr int kGroups = 4;  // upload_groups makes no more
   cudaStream_t cs = nullptr;
   cudaEvent_t start_ev = nullptr, ready[kGroups] = {};
   int c0[kGroups + 1] = {};
@@ -1723,14 +1716,9 @@ gp_ss_status gp_ss_loglik_grad_host(const gp_ss_model *m, const float *theta_hos
                     m->ch_first.size() == (size_t)m->n_series + 1 && m->h_meas3;
   float *d_meas3 = nullptr;
   if (pipe) {
-    std::vector<int> sb{0};
-    for (int g = 1; g < n_groups; ++g) {
-      const int64_t target = m->ev_off[m->n_series] * g / n_groups;
-      const int sp = (int)(std::lower_bound(m->ev_off.begin(), m->ev_off.end(), target) -
-                           m->ev_off.begin());
-      if (sp > sb.back() && sp < m->n_series) sb.push_back(sp);
-    }
-    sb.push_back(m->n_series);
+    const std::vector<int> sb =
+        gpss::upload_groups(m->ev_off.data(), m->ch_first.data(), m->n_series,
+                            (int64_t)m->n_sm * gpss::ELEM_BS);
     slices.n = (int)sb.size() - 1;
     // measurement records go up as 12-byte (y, r0, w) and are widened to the
     // kernels' float4 on the device (a quarter fewer bytes than the float4s)

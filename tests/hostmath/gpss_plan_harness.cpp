@@ -11,6 +11,13 @@ int ph_grad_segments(int product, int comb_prec, int D, int max_chunk, int ck, i
   return grad_segments({product != 0, comb_prec, D, D * (D + 1) / 2, max_chunk, ck, n_vch, n_sm});
 }
 
+int ph_upload_groups(const int64_t *ev_off, const int32_t *ch_first, int n_series,
+                     int64_t block_chunks, int *cut) {
+  const std::vector<int> c = upload_groups(ev_off, ch_first, n_series, block_chunks);
+  for (size_t i = 0; i < c.size(); ++i) cut[i] = c[i];
+  return (int)c.size() - 1;
+}
+
 // take_scratch against an allocator of `limit` bytes.  n[3], bytes: the lists
 // (needed, fast, plain) one after the other; held: bytes taken in the end;
 // got[i]: buffer i is in hand.  Returns 0 none, 1 plain, 2 fast.

@@ -4,6 +4,7 @@ import ctypes
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 HERE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "hostmath")
@@ -67,3 +68,34 @@ def test_scratch_is_refused_only_where_the_plain_way_does_not_fit(plan, needed, 
             assert held.value == with_plain
             assert list(got)[:len(flat) - len(plain)] == [1] * len(needed) + [0] * len(fast)
             assert all(list(got)[len(flat) - len(plain):])
+
+
+FULL = 152 * 128  # chunks of one block per multiprocessor
+
+
+@pytest.mark.parametrize("events,want", [
+    ([20000] * 1024, 4),            # 96 chunks each
+    ([200] * 2432, 4),              # many tiny series: 32 chunks each
+    ([200] * 2431, 3),
+    ([200] * 1216, 2),
+    ([200] * 1215, 1),
+    ([200] * 40, 1),
+    ([200000] + [40] * 5000, 2),    # the long series alone would hold 800 chunks
+    ([40] * 5000 + [200000], 2),
+    ([0] * 2000, 1),
+    ([100], 1),
+    ([0, 0], 1),
+])
+def test_upload_groups(plan, events, want):
+    n = len(events)
+    ev = np.concatenate([[0], np.cumsum(events)]).astype(np.int64)
+    ch = np.concatenate([[0], np.cumsum([32 * max(1, -(-e // 8192)) for e in events])])
+    ch = ch.astype(np.int32)
+    cut = (ctypes.c_int * 8)()
+    g = plan.ph_upload_groups(ctypes.c_void_p(ev.ctypes.data), ctypes.c_void_p(ch.ctypes.data),
+                              n, ctypes.c_int64(FULL), cut)
+    assert g == want
+    cut = list(cut)[:g + 1]
+    assert cut[0] == 0 and cut[-1] == n and cut == sorted(set(cut))
+    if g > 1:
+        assert min(np.diff(ch[cut])) >= FULL // 2
