@@ -387,13 +387,23 @@ GPSS_D void prod_prior(const ProdPar<SUM> &p, Dual2<float> (*m), Dual2<float> (*
   }
 }
 
+// Adds log S + e^2/S of an innovation e of variance S, and its tangent, in
+// FP64.  iS: the FP32 reciprocal of S, which two Newton steps bring to FP64
+// precision (one leaves 48 bits); three divisions took most of an event's time.
+GPSS_HD void prod_tally(double S, double dS, double e, double de, float iS, double &sum_ll,
+                        double &sum_d) {
+  double i = iS;
+  i = fma(i, fma(-S, i, 1.0), i);
+  i = fma(i, fma(-S, i, 1.0), i);
+  sum_ll += log(S) + e * e * i;
+  sum_d += i * (dS * (1.0 - e * e * i) + 2.0 * e * de);
+}
+
 // One event (instantaneous measurement y with variance r0) of the dual
 // product filter on the dense (m, P); adds log S + v^2/S and its tangent.
 //
 // Phi is block-diagonal (the product's Kronecker block, then the plain term):
-// the sums run over the blocks only.  The tangent's terms use S's reciprocal,
-// the FP32 one refined by a Newton step in FP64 (error 1e-14), in place of
-// three FP64 divisions, which took most of an event's time.
+// the sums run over the blocks only.
 template <bool SUM>
 GPSS_D void prod_event(const ProdPar<SUM> &p, const Osc2<Dual2<float>> &A,
                        const Osc2<Dual2<float>> &B, const Osc2<Dual2<float>> &C, float y, float r0,
@@ -477,11 +487,7 @@ GPSS_D void prod_event(const ProdPar<SUM> &p, const Osc2<Dual2<float>> &A,
 #pragma unroll
     for (int c = 0; c < D; ++c) P[r][c] = P[r][c] - u[r] * u[c] * iS;
   }
-  const double S = Sv.v, dS = Sv.da, e = vv.v, de = vv.da;
-  double iSd = iS.v;
-  iSd = iSd * (2.0 - S * iSd);
-  sum_ll += log(S) + e * e * iSd;
-  sum_d += iSd * (dS * (1.0 - e * e * iSd) + 2.0 * e * de);
+  prod_tally(Sv.v, Sv.da, vv.v, vv.da, iS.v, sum_ll, sum_d);
 }
 
 // One thread per (output row, parameter i) over the whole series (the plain

@@ -1,0 +1,49 @@
+"""FP64 parts of the device arithmetic, compiled for the host, against extended
+arithmetic."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "hostmath")
+ROOT = os.path.dirname(os.path.dirname(HERE))
+CSRC = os.path.join(ROOT, "paper_2601_02527_gb300", "csrc")
+EPS = 2.0 ** -53
+D = ctypes.c_double
+
+
+@pytest.fixture(scope="module")
+def lib():
+    src = os.path.join(HERE, "gpss_f64_harness.cu")
+    out = os.path.join(HERE, "_build", "libgpss_f64.so")
+    os.makedirs(os.path.dirname(out), exist_ok=True)
+    deps = [src] + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")]
+    if not os.path.exists(out) or os.path.getmtime(out) < max(map(os.path.getmtime, deps)):
+        tmp = out + f".tmp{os.getpid()}"
+        subprocess.check_call(["/usr/local/cuda/bin/nvcc", "-O2", "-std=c++17", "-Xcompiler",
+                               "-fPIC", "-shared", "-I", os.path.join(ROOT, "include"), "-I",
+                               CSRC, src, "-o", tmp])
+        os.replace(tmp, out)
+    lib = ctypes.CDLL(out)
+    lib.hf_prod_tally.argtypes = [D, D, D, D, ctypes.POINTER(D)]
+    return lib
+
+
+def test_product_sums_keep_double_precision(lib):
+    # at most eight roundings of half a unit each, of the terms' size
+    assert np.finfo(np.longdouble).eps < 2.0 ** -60
+    rng = np.random.default_rng(0)
+    L = np.longdouble
+    for _ in range(4000):
+        S = float(np.float32(np.exp(rng.uniform(-60, 60))))
+        e = float(np.float32(np.sqrt(S) * rng.standard_normal()))
+        dS = float(np.float32(S * rng.standard_normal() * 10.0 ** rng.uniform(-3, 3)))
+        de = float(np.float32(e * rng.standard_normal() * 10.0 ** rng.uniform(-3, 3)))
+        out = (D * 2)()
+        lib.hf_prod_tally(S, dS, e, de, out)
+        ll = [np.log(L(S)), L(e) * e / S]
+        d = [L(dS) / S, -L(e) * e * dS / (L(S) * S), 2 * L(e) * de / S]
+        assert abs(L(out[0]) - sum(ll)) <= 8 * EPS * sum(map(abs, ll))
+        assert abs(L(out[1]) - sum(d)) <= 8 * EPS * sum(map(abs, d))
