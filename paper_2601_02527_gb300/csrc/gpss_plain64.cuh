@@ -45,7 +45,15 @@ GPSS_HD double taylor64_entry(const double *c, int j, int k) {
   return s / (double)(j == 3 ? k + 3 : j == 4 ? k + 1 : k + 5);
 }
 
-// f's Taylor coefficients by its recurrence.
+// The unit of time T of a row's coefficients: a power of two within a factor of
+// two of 1/r.  In the caller's unit the last of them is of the size r^20 / 21!,
+// which leaves FP64's range for rates beyond about 1e17 or 1e-17; in this one
+// every entry is of order one at most.  Scaling by it is exact.
+GPSS_HD double taylor64_unit(double r2) {
+  return r2 > 0.0 && isfinite(r2) ? ldexp(1.0, -(ilogb(r2) >> 1)) : 1.0;
+}
+
+// f's Taylor coefficients by its recurrence, from a T and w2 T^2.
 GPSS_HD void taylor64_c(double a, double w2, double *c) {
   c[0] = 0.0;
   c[1] = 1.0;
@@ -54,13 +62,17 @@ GPSS_HD void taylor64_c(double a, double w2, double *c) {
     c[n + 2] = -(2.0 * a * (n + 1) * c[n + 1] + w2 * c[n]) / (double)((n + 2) * (n + 1));
 }
 
+// A row's table: the entries of the six scalars, then 1/T.
+constexpr int TAB64_LEN = 6 * TAB64_N + 1;
+
 GPSS_HD Disc<double> disc_tab64(double t, const double *tab) {
   double g[6];
+  const double u = t * tab[6 * TAB64_N];
 #pragma unroll
   for (int j = 0; j < 6; ++j) g[j] = tab[j * TAB64_N + TAB64_N - 1];
   for (int k = TAB64_N - 2; k >= 0; --k)
 #pragma unroll
-    for (int j = 0; j < 6; ++j) g[j] = fma(g[j], t, tab[j * TAB64_N + k]);
+    for (int j = 0; j < 6; ++j) g[j] = fma(g[j], u, tab[j * TAB64_N + k]);
   const double t2 = t * t, t3 = t2 * t;
   return Disc<double>{g[0] * t, g[1], g[2] * t2, g[3] * t3, g[4] * t, g[5] * (t3 * t2)};
 }
@@ -153,7 +165,7 @@ __global__ void __launch_bounds__(64) k_plain64(DevModel M, const float *__restr
   __shared__ double rec[2][32][R::LEN];
   __shared__ double Sb[2][32], vb[2][32];
   __shared__ uint8_t tg[2][32];
-  __shared__ double tab[NT][6 * TAB64_N];
+  __shared__ double tab[NT][TAB64_LEN];
   __shared__ double cs[NT][TAB64_N + 2];
   __shared__ double Pm[NE], T[NE];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -166,7 +178,11 @@ __global__ void __launch_bounds__(64) k_plain64(DevModel M, const float *__restr
   if (threadIdx.x < NT) {
 #pragma unroll
     for (int t = 0; t < NT; ++t)
-      if (t == (int)threadIdx.x) taylor64_c(tc[t].a, tc[t].w2, cs[t]);
+      if (t == (int)threadIdx.x) {
+        const double unit = taylor64_unit(tc[t].r2);
+        tab[t][6 * TAB64_N] = 1.0 / unit;
+        taylor64_c(tc[t].a * unit, tc[t].w2 * unit * unit, cs[t]);
+      }
   }
   if (threadIdx.x == 0) {
     // P0 = blkdiag(P_inf, I), m0 = 0

@@ -13,4 +13,22 @@ void hf_prod_tally(double S, double dS, double e, double de, double *out2) {
   prod_tally(S, dS, e, de, 1.0f / (float)S, out2[0], out2[1]);
 }
 
+// The plain FP64 filter's step scalars (f, f', F1, I_ff, I_pp, I_FF).
+void hf_plain64_scalars(double t, double a, double beta, double *out6) {
+  TermC<double> c;
+  c.a = a;
+  c.beta = beta;
+  c.w2 = beta + a * a;
+  c.qc = c.var = 1.0;
+  finish_termc(c);
+  double cs[TAB64_N + 2], tab[TAB64_LEN];
+  const double T = taylor64_unit(c.r2);
+  tab[6 * TAB64_N] = 1.0 / T;
+  taylor64_c(c.a * T, c.w2 * T * T, cs);
+  for (int e = 0; e < 6 * TAB64_N; ++e) tab[e] = taylor64_entry(cs, e / TAB64_N, e % TAB64_N);
+  const Disc<double> d = discretize_tab64(t, c, tab);
+  const double v[6] = {d.f, d.fp, d.F1, d.Iff, d.Ipp, d.IFF};
+  for (int i = 0; i < 6; ++i) out6[i] = v[i];
+}
+
 }  // extern "C"

@@ -28,6 +28,7 @@ def lib():
         os.replace(tmp, out)
     lib = ctypes.CDLL(out)
     lib.hf_prod_tally.argtypes = [D, D, D, D, ctypes.POINTER(D)]
+    lib.hf_plain64_scalars.argtypes = [D, D, D, ctypes.POINTER(D)]
     return lib
 
 
@@ -47,3 +48,22 @@ def test_product_sums_keep_double_precision(lib):
         d = [L(dS) / S, -L(e) * e * dS / (L(S) * S), 2 * L(e) * de / S]
         assert abs(L(out[0]) - sum(ll)) <= 8 * EPS * sum(map(abs, ll))
         assert abs(L(out[1]) - sum(d)) <= 8 * EPS * sum(map(abs, d))
+
+
+@pytest.mark.parametrize("q", [0.2, 0.5, 0.7, 8.0])
+@pytest.mark.parametrize("x", [1e-3, 0.3, 0.99, 1.7, 30.0])  # omega0 t: Taylor and closed branches
+@pytest.mark.parametrize("k", [-120, -60, -7, 7, 60, 120])
+def test_plain64_scalars_in_any_unit_of_time(lib, q, x, k):
+    # times in units of 2^k: every scalar scales by a power of two, exactly
+    def scalars(u):
+        w0 = 0.7 / u
+        a = w0 / (2 * q)
+        beta = 0.0 if q == 0.5 else w0 * w0 * (1 - 1 / (4 * q * q))
+        out = (D * 6)()
+        lib.hf_plain64_scalars(x / w0, a, beta, out)
+        return np.array(out)
+
+    u = 2.0 ** k
+    one = scalars(1.0)
+    assert np.all(np.isfinite(one)) and np.all(one[3:] > 0)  # the integrals of squares
+    assert np.array_equal(scalars(u), one * [u, 1.0, u ** 2, u ** 3, u, u ** 5])
