@@ -18,6 +18,8 @@
 // (k_prod_grad, schedule 3).
 #pragma once
 
+#include <cstdint>
+#include <cstring>
 #include <type_traits>
 
 #include "gpss_kernels.cuh"
@@ -68,8 +70,8 @@ GPSS_HD Osc2<T> osc2(F dt, T w0, T Q, T var) {
 // every parameter's thread in the gradient).  Per lane-step and oscillator
 // one float4 (f, f', I_ff, I_pp), oscillator j of step k of the chunk on lane
 // l of warp w at ((w_doff[w] + 32 k) NO + 32 j + l); with tangents, two more
-// float4 (d/da, d/dbeta of the four) behind all sets' values, in the same
-// order.  150 series of 500 to 5000 instants with the gradient, product +
+// float4 (s d/da, s^2 d/dbeta of the four, s = prod_unit) in an array of their
+// own, in the same order.  150 series of 500 to 5000 instants with the gradient, product +
 // Matern-3/2: scalars 67 us, elements 442 -> 121 us, gradient 1099 -> 304 us.
 // ---------------------------------------------------------------------------
 template <bool SUM>
@@ -98,6 +100,48 @@ GPSS_D bool prod_overdamped(const DevModel &M, const float *th) {
   return th[2] < 0.5f || th[4] < 0.5f || (SUM && M.kinds[1] == 1 && th[7] < 0.5f);
 }
 
+// Unit of rate of an oscillator's tangents, a power of two within a factor of
+// two of omega0.  d/da and d/dbeta themselves are of the size t and t^2 times
+// the scalar (I_ff: t^3), which FP32 does not hold where t is 1e7 or 1e-7 of
+// the caller's unit; scaling by a power of two is exact.
+GPSS_HD float prod_unit(float w0) {
+  uint32_t b;
+  memcpy(&b, &w0, sizeof b);
+  b &= 0x7f800000u;  // the exponent; the least normal number for denormals
+  if (b == 0u) b = 0x00800000u;
+  if (b == 0x7f800000u) return 1.f;
+  float s;
+  memcpy(&s, &b, sizeof s);
+  return s;
+}
+
+// Tangents of a step's scalars (f, f', I_ff, I_pp), in that unit: formed with
+// time in units of 1/s, where the duals' seeds are ones, and scaled back.
+GPSS_HD void prod_tangents(float dt, float a, float beta, float s, float4 &ta, float4 &tb) {
+  using T = Dual2<float>;
+  const float is = 1.f / s, is3 = is * is * is;
+  const Disc<T> e =
+      discretize<T, float, true>(dt * s, mk(a * is, 1.f, 0.f), mk(beta * is * is, 0.f, 1.f));
+  ta = make_float4(e.f.da * is, e.fp.da, e.Iff.da * is3, e.Ipp.da * is);
+  tb = make_float4(e.f.db * is, e.fp.db, e.Iff.db * is3, e.Ipp.db * is);
+}
+
+// The scalars with the tangent of a parameter whose rates change by (da, db)
+// in that unit (prod_rates_tangent).
+GPSS_HD Disc<Dual2<float>> prod_dual(float4 q, float4 ta, float4 tb, float2 dr) {
+  Disc<Dual2<float>> d;
+  d.f = mk(q.x, ta.x * dr.x + tb.x * dr.y, 0.f);
+  d.fp = mk(q.y, ta.y * dr.x + tb.y * dr.y, 0.f);
+  d.Iff = mk(q.z, ta.z * dr.x + tb.z * dr.y, 0.f);
+  d.Ipp = mk(q.w, ta.w * dr.x + tb.w * dr.y, 0.f);
+  d.F1 = d.IFF = mk(0.f, 0.f, 0.f);
+  return d;
+}
+GPSS_HD float2 prod_rates_tangent(Dual2<float> a, Dual2<float> beta, float w0) {
+  const float is = 1.f / prod_unit(w0);
+  return make_float2(a.da * is, beta.da * is * is);
+}
+
 GPSS_D size_t prod_col(const DevModel &M, int set, int c) {
   return (size_t)set * M.dcache_steps + M.w_doff[c >> 5];
 }
@@ -117,6 +161,7 @@ __global__ void __launch_bounds__(128) k_prod_scalars(DevModel M, const float *_
   F w0, Q, a, beta;
   prod_osc<SUM>(M, theta + (size_t)(per_series ? M.ch_series[c] : set) * M.n_params, j, w0, Q);
   osc_rates<F, F>(w0, Q, a, beta);
+  const F unit = prod_unit(w0);
   const size_t col = prod_col(M, set, c);
   for (int k = k0; k < k1; ++k) {
     const F dt = __ldg(M.ilv + lane_step(M, c, k)).x;
@@ -124,11 +169,8 @@ __global__ void __launch_bounds__(128) k_prod_scalars(DevModel M, const float *_
     const size_t at = (col + (size_t)k * 32) * NO + 32 * j + lane;
     sc[at] = make_float4(d.f, d.fp, d.Iff, d.Ipp);
     if (tan) {
-      using T = Dual2<F>;
-      const Disc<T> e = discretize<T, F, true>(dt, mk(a, F(1), F(0)), mk(beta, F(0), F(1)));
       const size_t t0 = (col + (size_t)k * 32) * (2 * NO) + 64 * j + lane;
-      tan[t0] = make_float4(e.f.da, e.fp.da, e.Iff.da, e.Ipp.da);
-      tan[t0 + 32] = make_float4(e.f.db, e.fp.db, e.Iff.db, e.Ipp.db);
+      prod_tangents(dt, a, beta, unit, tan[t0], tan[t0 + 32]);
     }
   }
 }
@@ -145,17 +187,9 @@ GPSS_D Disc<float> prod_load(const float4 *rec, int j) {
   return d;
 }
 
-// ... with the tangent of the thread's parameter, (a.da, beta.da).
-GPSS_D Disc<Dual2<float>> prod_load_dual(const float4 *rec, const float4 *trec, int j, float da,
-                                         float db) {
-  const float4 q = __ldg(rec + 32 * j), ta = __ldg(trec + 64 * j), tb = __ldg(trec + 64 * j + 32);
-  Disc<Dual2<float>> d;
-  d.f = mk(q.x, ta.x * da + tb.x * db, 0.f);
-  d.fp = mk(q.y, ta.y * da + tb.y * db, 0.f);
-  d.Iff = mk(q.z, ta.z * da + tb.z * db, 0.f);
-  d.Ipp = mk(q.w, ta.w * da + tb.w * db, 0.f);
-  d.F1 = d.IFF = mk(0.f, 0.f, 0.f);
-  return d;
+// ... with the tangent of the thread's parameter.
+GPSS_D Disc<Dual2<float>> prod_load_dual(const float4 *rec, const float4 *trec, int j, float2 dr) {
+  return prod_dual(__ldg(rec + 32 * j), __ldg(trec + 64 * j), __ldg(trec + 64 * j + 32), dr);
 }
 
 template <bool SUM>
@@ -570,7 +604,8 @@ __global__ void __launch_bounds__(64) k_prod_grad_chunk(DevModel M, const float 
   const int row = per_series ? s : set;
   const int orow = per_series ? s : set * M.n_series + s;
   const uint8_t flags = M.ch_flags[c];
-  const ProdPar<SUM> p = prod_par<SUM>(M, theta + (size_t)row * np, ip);
+  const float *th = theta + (size_t)row * np;
+  const ProdPar<SUM> p = prod_par<SUM>(M, th, ip);
   T m[D], P[D][D];
   if (flags & 1) {
     prod_prior<SUM>(p, m, P);
@@ -592,6 +627,18 @@ __global__ void __launch_bounds__(64) k_prod_grad_chunk(DevModel M, const float 
   osc_rates<T, F>(p.wb, p.qb, ab, bb);
   osc_rates<T, F>(p.wc, p.qcq, ac, bc);
   const T one = cst<T>(F(1)), varc = p.sc * p.sc;
+  // the records' units come from the rates as k_prod_scalars forms them: a dual
+  // quotient may round to the other side of a power of two
+  F w0, Q;
+  prod_osc<SUM>(M, th, 0, w0, Q);
+  const float2 da = prod_rates_tangent(aa, ba, w0);
+  prod_osc<SUM>(M, th, 1, w0, Q);
+  const float2 db = prod_rates_tangent(ab, bb, w0);
+  float2 dc{};
+  if constexpr (SUM) {
+    prod_osc<SUM>(M, th, 2, w0, Q);
+    dc = prod_rates_tangent(ac, bc, w0);
+  }
   const size_t col = prod_col(M, set, c);
   const float4 *rec = sc ? sc + col * NO + (c & 31) : nullptr;
   const float4 *trec = sc ? tan + col * (2 * NO) + (c & 31) : nullptr;
@@ -600,10 +647,10 @@ __global__ void __launch_bounds__(64) k_prod_grad_chunk(DevModel M, const float 
     const float4 q = __ldg(M.ilv + lane_step(M, c, k));  // (dt, y, yerr^2, 1)
     Osc2<T> A, B, C{};
     if (rec) {
-      A = osc2_of<T, F>(prod_load_dual(rec, trec, 0, aa.da, ba.da), aa, p.wa, p.qa, one);
-      B = osc2_of<T, F>(prod_load_dual(rec, trec, 1, ab.da, bb.da), ab, p.wb, p.qb, p.var);
+      A = osc2_of<T, F>(prod_load_dual(rec, trec, 0, da), aa, p.wa, p.qa, one);
+      B = osc2_of<T, F>(prod_load_dual(rec, trec, 1, db), ab, p.wb, p.qb, p.var);
       if constexpr (SUM)
-        C = osc2_of<T, F>(prod_load_dual(rec, trec, 2, ac.da, bc.da), ac, p.wc, p.qcq, varc);
+        C = osc2_of<T, F>(prod_load_dual(rec, trec, 2, dc), ac, p.wc, p.qcq, varc);
       rec += 32 * NO;
       trec += 64 * NO;
     } else {

@@ -1,5 +1,5 @@
-"""FP64 parts of the device arithmetic, compiled for the host, against extended
-arithmetic."""
+"""Parts of the device arithmetic, compiled for the host: FP64 sums against
+extended arithmetic, and step scalars in any unit of time."""
 import ctypes
 import os
 import subprocess
@@ -29,6 +29,8 @@ def lib():
     lib = ctypes.CDLL(out)
     lib.hf_prod_tally.argtypes = [D, D, D, D, ctypes.POINTER(D)]
     lib.hf_plain64_scalars.argtypes = [D, D, D, ctypes.POINTER(D)]
+    f = ctypes.c_float
+    lib.hf_prod_dual.argtypes = [f, f, f, ctypes.c_int, ctypes.POINTER(D)]
     return lib
 
 
@@ -67,3 +69,23 @@ def test_plain64_scalars_in_any_unit_of_time(lib, q, x, k):
     one = scalars(1.0)
     assert np.all(np.isfinite(one)) and np.all(one[3:] > 0)  # the integrals of squares
     assert np.array_equal(scalars(u), one * [u, 1.0, u ** 2, u ** 3, u, u ** 5])
+
+
+@pytest.mark.parametrize("q", [0.2, 0.5, 0.7, 8.0])
+@pytest.mark.parametrize("x", [0.1, 1.1, 1.7, 30.0])
+@pytest.mark.parametrize("which", [0, 1])
+@pytest.mark.parametrize("k", [-24, -10, 10, 24])
+def test_product_tangents_in_any_unit_of_time(lib, q, x, which, k):
+    # FP32 scalars and the tangent with respect to omega0 or Q scale by powers
+    # of two, exactly (d I_ff / d omega0 is of the size 2^(4 k))
+    def scalars(u):
+        out = (D * 8)()
+        w0 = float(np.float32(0.7)) / u
+        lib.hf_prod_dual(float(np.float32(x / 0.7)) * u, w0, q, which, out)
+        return np.array(out)
+
+    u = 2.0 ** k
+    one = scalars(1.0)
+    assert np.all(np.isfinite(one)) and np.all(one[4:6] != 0)
+    size = np.array([u, 1.0, u ** 3, u])
+    assert np.array_equal(scalars(u), one * np.concatenate([size, size * (u if which == 0 else 1)]))
