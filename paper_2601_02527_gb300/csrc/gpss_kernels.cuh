@@ -641,13 +641,18 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
   // chunks [c_begin, c_begin + c_count) of every parameter set (a multiple of
   // 32 chunks per series keeps each warp in one series)
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= (n_vch / M.n_chunks) * c_count) return;
+  const int cw = (c_count + 31) & ~31;
+  if (l >= (n_vch / M.n_chunks) * cw) return;
   int set, c;
+  bool live = true;
   if (c_count == M.n_chunks) {
     c = chunk_of_thread(M, n_vch, l, set);
   } else {
-    set = l / c_count;
-    c = c_begin + l % c_count;
+    // a part of the chunks (any part of a series split in time): whole warps
+    // of one parameter row, whose lanes past its end only help to stage the table
+    set = l / cw;
+    live = l % cw < c_count;
+    c = c_begin + min(l % cw, c_count - 1);
   }
   const int vc = set * M.n_chunks + c;
   const int s = M.ch_series[c];
@@ -664,7 +669,7 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
   const int k_lo = seg < 0 ? 0 : k_hi - ck;
   const float4 *tab =
       stage_table<S::NT>(tabs, row, smem_tab + (threadIdx.x >> 5) * (S::NT * TAB_TERM / 4));
-  if (seg >= 0 && k_lo <= 0) return;  // nothing precedes the first segment
+  if (!live || (seg >= 0 && k_lo <= 0)) return;  // nothing precedes the first segment
   auto body = [&](auto od_tag) {
     constexpr bool OD = decltype(od_tag)::value;
     const bool first = seg < 0 && (M.ch_flags[c] & 1);
@@ -2122,7 +2127,7 @@ cudaError_t launch_elem(const DevModel &M, const float *theta, int n_vch, int pe
   if (pck && (ck < 2 || ck > 64 || (ck & 1))) return cudaErrorInvalidValue;
   const int bs = ELEM_BS;
   const size_t smem = (size_t)(bs / 32) * S::NT * TAB_TERM * sizeof(float);
-  const int64_t nt = (int64_t)(n_vch / M.n_chunks) * c_count;
+  const int64_t nt = (int64_t)(n_vch / M.n_chunks) * ((c_count + 31) & ~31);
   // every segment's own element but the first one's beside the chunks'
   const dim3 nb((unsigned)((nt + bs - 1) / bs), segel ? n_seg : 1);
   k_elem<S><<<nb, bs, smem, st>>>(M, theta, n_vch, per_series, ef, ed, err, tabs, pck,
