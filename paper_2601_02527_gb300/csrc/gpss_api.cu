@@ -1116,6 +1116,7 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
       // tangents); without them every thread forms its own step by step
       const size_t bytes = rows * (size_t)m->dcache_steps * (o.D / 2) * sizeof(float4);
       if (m->step_cache == 0 && m->max_chunk <= 65535 * gpss::PROD_STEPS &&
+          gpss::prod_scalars_at_once(grad, m->n_terms > 1, m->max_chunk, n_vch, m->n_sm) &&
           bytes * (grad ? 3 : 1) <= kDcacheMax) {
         put(fast, dcache, bytes);
         if (grad) put(fast, ptan, 2 * bytes);

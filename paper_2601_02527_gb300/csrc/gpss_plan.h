@@ -52,6 +52,26 @@ inline int grad_segments(const SegmentCase &c) {
   return replay_bytes(c.ck, c.D, c.NP, c.n_vch, n_seg) <= kMaxReplay ? n_seg : 1;
 }
 
+// Whether a product model's step scalars are formed for all steps at once
+// rather than by the chunks' threads.  For a gradient always: every
+// parameter's thread reads them (150 series of 500 to 5000 instants 1633 ->
+// 642 us; one of 100: 92 -> 86 us).  The log-likelihood alone reads each once:
+// they shorten a chunk's serial chain but cost a pass over memory and two
+// launches, so they are formed where chunks are long and warps of chunks too
+// few to hide the chain.  Product alone (two oscillators), at once against
+// step by step, 152 SMs: 30 warps, chunks of 32 events 72 us against 77, of 64
+// 91 against 116; 304 warps, 64 events 108 against 116; 608 warps, 64 events
+// 128 against 120, 250 events 435 against 397.  With a plain term (three): 30
+// warps, 8 events 74 against 75, 32 events 95 against 140; 608 warps, 32 events
+// 130 against 159; 912 warps 32 events 153 against 163, 128 events 464 against
+// 454.  Rows with an overdamped factor, whose elements form their own, pay 7 to
+// 10 us for the launches that skip them, which is why the shorter chunks
+// with a small gain are left out (64 and 32 events: 2 to 7 % of such a call).
+inline bool prod_scalars_at_once(bool grad, bool plain_term, int max_chunk, int n_vch, int n_sm) {
+  if (grad) return true;
+  return max_chunk >= (plain_term ? 32 : 64) && n_vch / 32 <= (plain_term ? 4 : 2) * n_sm;
+}
+
 // First series of each group in which a re-sent event stream goes up, and the
 // number of series at the end.  A group's element pass takes at least its
 // longest chunk's serial time however few chunks it has, so groups hold

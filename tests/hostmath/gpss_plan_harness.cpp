@@ -11,6 +11,10 @@ int ph_grad_segments(int product, int comb_prec, int D, int max_chunk, int ck, i
   return grad_segments({product != 0, comb_prec, D, D * (D + 1) / 2, max_chunk, ck, n_vch, n_sm});
 }
 
+int ph_prod_scalars(int grad, int plain_term, int max_chunk, int n_vch, int n_sm) {
+  return prod_scalars_at_once(grad != 0, plain_term != 0, max_chunk, n_vch, n_sm);
+}
+
 int ph_upload_groups(const int64_t *ev_off, const int32_t *ch_first, int n_series,
                      int64_t block_chunks, int *cut) {
   const std::vector<int> c = upload_groups(ev_off, ch_first, n_series, block_chunks);

@@ -99,3 +99,14 @@ def test_upload_groups(plan, events, want):
     assert cut[0] == 0 and cut[-1] == n and cut == sorted(set(cut))
     if g > 1:
         assert min(np.diff(ch[cut])) >= FULL // 2
+
+
+@pytest.mark.parametrize("case,want", [
+    ((1, 0, 1, 32, 152), 1), ((1, 1, 4, 10 ** 6 * 32, 152), 1),  # gradients: always
+    ((0, 0, 64, 32, 152), 1), ((0, 0, 63, 32, 152), 0),
+    ((0, 0, 64, 32 * 304, 152), 1), ((0, 0, 64, 32 * 305, 152), 0),
+    ((0, 1, 32, 32, 152), 1), ((0, 1, 31, 32, 152), 0),
+    ((0, 1, 32, 32 * 608, 152), 1), ((0, 1, 32, 32 * 609, 152), 0),
+])
+def test_product_scalars_at_once(plan, case, want):
+    assert plan.ph_prod_scalars(*case) == want
