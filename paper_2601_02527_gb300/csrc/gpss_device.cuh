@@ -637,8 +637,6 @@ GPSS_HD DF operator*(DF x, DF y) {
   e = fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, e));
   return df_fast(p, e);
 }
-GPSS_HD Dual2<DF> mkdf(DF v, DF da, DF db) { return Dual2<DF>{v, da, db}; }
-GPSS_HD Dual2<DF> operator*(Dual2<DF> x, DF c) { return mkdf(x.v * c, x.da * c, x.db * c); }
 
 // Table coefficients with the scale of the table's range T taken out, in
 // double-float (the form the table kernel computes; FP64 inputs, FP32 pipe).
@@ -679,7 +677,8 @@ GPSS_HD void taylor_cg_scaled(const TabConst &K, const DF *rcp, DF *c, DF *g) {
   for (int n = 1; n + 2 <= TAB_NCF; ++n)
     c[n + 2] = taylor_step(K.aT * df_int(2 * (n + 1)), c[n + 1], K.w2T2, c[n],
                            rcp[n + 2] * rcp[n + 1]);
-  for (int n = 1; n + 1 <= TAB_NCF; ++n) g[n + 1] = taylor_step(K.aT, g[n], K.hT2, c[n - 1], rcp[n + 1]);
+  for (int n = 1; n + 1 <= TAB_NCF; ++n)
+    g[n + 1] = taylor_step(K.aT, g[n], K.hT2, c[n - 1], rcp[n + 1]);
 }
 
 // Coefficients n of F1 = int f (times t^{n+1}) and its tangents.
@@ -1320,7 +1319,6 @@ GPSS_HD void obs_project_tag(uint8_t tag, F w, const F *m, const F *P, F *u, F &
   obs_project<S>((tag >> 1) & 7, w, m, P, u, hu, hm);
 }
 
-// Load per-term constants and s^2 from a row of natural parameters.
 // a, beta of term t alone (the table kernel's inputs).
 template <int NT>
 GPSS_HD void load_rates(const float *th, const int *kinds, int t, double &a, double &beta) {
@@ -1334,6 +1332,7 @@ GPSS_HD void load_rates(const float *th, const int *kinds, int t, double &a, dou
   beta = (q == 0.5) ? 0.0 : w0 * w0 * (1.0 - 1.0 / (4.0 * q * q));
 }
 
+// Load per-term constants and s^2 from a row of natural parameters.
 template <int NT, class F>
 GPSS_HD void load_terms(const float *th, const int *kinds, TermC<F> *tc, F &s2) {
   int j = 0;

@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(ELEM_BS, ELEM_MIN_BLOCKS) k_elem(DevModel M, c
     ed[(size_t)n_vch + vc] = ld;
     ed[(size_t)2 * n_vch + vc] = (double)n_end;
     if (bad) flag_error(err, orow, 7);
-};
+  };
   // rows with an overdamped term, and every row of a mixed model, take the
   // general body, the others the lean one (whole warps: a warp's chunks share
   // one row)
@@ -1510,9 +1510,10 @@ __global__ void __launch_bounds__(64) k_seg_adjoint(DevModel M, int n_vch,
 // coalesced across the warp; slot k holds (m, P) before the segment's k-th
 // event), then walked backwards in time.  With seg_adj set (the adjoints at
 // segment ends, k_seg_adjoint), blockIdx.y picks the thread's only segment,
-// counted from the chunk's end.  With gdt set, the walk also writes, per event k of theta set r, gdt[r n_events + k] = d loglik / d
-// (gap before k) and, at an end event, gwe[...] = w^2 d loglik / d w
-// (w = 1/delta of its measurement; dw/dt_start = w^2 = -dw/dt_end).
+// counted from the chunk's end.  With gdt set, the walk also writes, per event
+// k of theta set r, gdt[r n_events + k] = d loglik / d (gap before k) and, at
+// an end event, gwe[...] = w^2 d loglik / d w (w = 1/delta of its measurement;
+// dw/dt_start = w^2 = -dw/dt_end).
 template <class S>
 __global__ void __launch_bounds__(GRAD_BS, GRAD_MIN_BLOCKS) k_grad(DevModel M, const float *__restrict__ theta, int n_vch,
                                              int per_series, const void *__restrict__ state_end,

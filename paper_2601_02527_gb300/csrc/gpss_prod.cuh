@@ -701,8 +701,8 @@ cudaError_t launch_prod_grad_chunk(const DevModel &M, const float *theta, int n_
   const int bs = 64;
   const int64_t nt = (int64_t)n_vch * M.n_params;
   k_prod_grad_chunk<SUM, ES><<<(unsigned)((nt + bs - 1) / bs), bs, 0, st>>>(
-      M, theta, n_vch, per_series, state_end, se64, adj_end, gpart, err, reinterpret_cast<const float4 *>(sc),
-      reinterpret_cast<const float4 *>(tan));
+      M, theta, n_vch, per_series, state_end, se64, adj_end, gpart, err,
+      reinterpret_cast<const float4 *>(sc), reinterpret_cast<const float4 *>(tan));
   GPSS_COUNT_LAUNCH();
   return cudaGetLastError();
 }

@@ -741,7 +741,8 @@ cudaError_t scan_elems(const T *src, int n, T *dst, int mode, int rev_index, int
   GPSS_COUNT_LAUNCH();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  e = scan_elems<S, T>(agg, nt, aggscan, 0, 0, rev_op, aggscan + (size_t)Elem<S>::NF * nt, n_sm, st);
+  e = scan_elems<S, T>(agg, nt, aggscan, 0, 0, rev_op, aggscan + (size_t)Elem<S>::NF * nt, n_sm,
+                       st);
   if (e != cudaSuccess) return e;
   tiles(aggscan, nt);
   GPSS_COUNT_LAUNCH();
@@ -844,7 +845,8 @@ __global__ void __launch_bounds__(32 * COOP) k_warp_scan_coop(const float *__res
   for (int f = threadIdx.x >> 5; f < NF; f += COOP)
     out[(size_t)f * n_vch + vc] = buf[at][(threadIdx.x & 31) * ST + f];
   if (dir == 0)
-    for (int f = threadIdx.x; f < NF; f += 32 * COOP) wtot[(size_t)f * n_w + w] = buf[at][31 * ST + f];
+    for (int f = threadIdx.x; f < NF; f += 32 * COOP)
+      wtot[(size_t)f * n_w + w] = buf[at][31 * ST + f];
 }
 
 // Per chunk: filtered end state = (state entering the warp) o (warp-local
