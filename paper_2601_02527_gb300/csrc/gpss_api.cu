@@ -1077,11 +1077,11 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
     // every recomputation segment but a chunk's first
     const int ck = m->ckpt_interval;
     const int n_pck = std::max((m->max_chunk - 1) / ck, 1);
-    int n_seg = grad && tree && !dexp && !pred
-                    ? gpss::grad_segments({m->product, m->comb_prec, o.D, o.NP, m->max_chunk, ck,
-                                           n_vch, m->n_sm})
-                    : 1;
     const size_t nv = (size_t)n_vch, n_w = nv / 32, rows = nv / m->n_chunks;
+    int n_seg = 1;
+    if (grad && tree && !dexp && !pred)
+      n_seg = gpss::grad_segments({m->product, m->comb_prec, o.D, o.NP, m->max_chunk, ck, n_vch,
+                                   (int64_t)rows * m->dcache_steps, m->n_sm});
     const size_t exp_ev = (size_t)(per_series ? 1 : n_sets) * m->n_events;
     const size_t part = m->n_params * nv * sizeof(float);
     std::vector<gpss::Buffer> needed, fast, plain;

@@ -17,6 +17,7 @@ struct SegmentCase {
   int max_chunk;  // events of the longest chunk
   int ck;         // events per segment
   int n_vch;      // chunks of the call (all parameter sets)
+  int64_t steps;  // lane-steps of their warps: 32 x each warp's longest chunk
   int n_sm;       // multiprocessors
 };
 
@@ -29,18 +30,22 @@ inline size_t replay_bytes(int ck, int D, int NP, int n_vch, int n_seg) {
 // thread each (1: one thread per chunk walks them in turn).  A thread takes
 // the serial time of its events, so too few chunks leave the GPU idle;
 // parallel segments cost each segment's own element beside the chunk's and a
-// boundary adjoint per segment.  The line lies where both take the same time:
-// 6 warps of chunks per SM, 12 for states of at most 4 (cheaper elements).
-// One call, parallel against in turn, 152 SMs: two SHO terms 911 warps 1254
-// us against 1367, 1215 warps 1534 against 1418; SHO + Matern-3/2 with three
-// slots 624 warps 1674 against 1935, 936 warps 2136 each; instants 1205
-// warps 1009 against 1152, 1649 warps 1279 against 1300.  The adjoint at a
-// segment's end differs from the walked one in rounding; exposure gradients
-// and predictions, differences of nearly equal terms, would show it at 3e-5
-// of their size and keep the walk in turn.  The segments' elements and the
-// information carried back through them are FP32: a model whose combination
-// runs in FP64 starts the walk in turn from the FP64 adjoint at the chunk's
-// end and keeps it.
+// boundary adjoint per segment.  The line lies where both take the same time,
+// which for chunks of one length is 1000 to 1100 warps of them on 152 SMs: two
+// SHO terms 912 warps 1132 us against 1233, 1064 warps 1311 against 1253; SHO +
+// Matern-3/2 on instants 912 warps 942 against 1094, 1216 warps 1263 against
+// 1153, 1824 warps 1787 against 1361; SHO alone 912 warps 541 against 597, 1216
+// warps 683 against 637.  Where lengths differ the work counts, not the warps:
+// with as many steps as 836 (1043) warps of the longest chunk have, 1306 (1616)
+// warps of instants took 995 us against 1145 (1195 against 1214), SHO alone 561
+// against 617 (639 against 659).  So: up to 6 warps of chunks per SM, or for
+// states of at most 4 up to 12 that have no more steps than 7 of the longest.
+// The adjoint at a segment's end differs from the walked one in rounding;
+// exposure gradients and predictions, differences of nearly equal terms, would
+// show it at 3e-5 of their size and keep the walk in turn.  The segments'
+// elements and the information carried back through them are FP32: a model
+// whose combination runs in FP64 starts the walk in turn from the FP64 adjoint
+// at the chunk's end and keeps it.
 inline int grad_segments(const SegmentCase &c) {
   constexpr int kMaxSegments = 1024;  // k_seg_info carries the adjoints back through them in turn
   constexpr size_t kMaxReplay = (size_t)2 << 30;  // bytes of the replay buffers
@@ -49,6 +54,7 @@ inline int grad_segments(const SegmentCase &c) {
   const int n_seg = (c.max_chunk + c.ck - 1) / c.ck;
   const int per_sm = c.D <= 4 ? 12 : 6;
   if (c.n_vch / 32 > per_sm * c.n_sm || n_seg < 2 || n_seg > kMaxSegments) return 1;
+  if (c.steps > (int64_t)32 * c.max_chunk * 7 * c.n_sm) return 1;
   return replay_bytes(c.ck, c.D, c.NP, c.n_vch, n_seg) <= kMaxReplay ? n_seg : 1;
 }
 

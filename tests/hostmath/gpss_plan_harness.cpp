@@ -6,9 +6,10 @@ using namespace gpss;
 
 extern "C" {
 
-int ph_grad_segments(int product, int comb_prec, int D, int max_chunk, int ck, int n_vch,
-                     int n_sm) {
-  return grad_segments({product != 0, comb_prec, D, D * (D + 1) / 2, max_chunk, ck, n_vch, n_sm});
+int ph_grad_segments(int product, int comb_prec, int D, int max_chunk, int ck, int n_vch, int n_sm,
+                     int64_t steps) {
+  return grad_segments(
+      {product != 0, comb_prec, D, D * (D + 1) / 2, max_chunk, ck, n_vch, steps, n_sm});
 }
 
 int ph_prod_scalars(int grad, int plain_term, int max_chunk, int n_vch, int n_sm) {

@@ -52,3 +52,21 @@ def test_fp64_combination_walks_in_turn(terms, prec):
     assert abs(ll.item() - ref_ll) <= 1e-4 * max(abs(ref_ll), 70.0)
     g = g[0].cpu().numpy().astype(np.float64)
     assert np.all(np.abs(g - ref) <= 1e-3 * np.abs(ref) + 1e-4 * np.abs(ref).max())
+
+
+@pytest.mark.parametrize("full,parallel", [(5, True), (8, False)])
+def test_equal_chunks_past_the_line_walk_in_turn(full, parallel):
+    # states of 3, `full` warps per SM of chunks of 64 events each
+    import paper_2601_02527_gb300 as gp
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n, rows = 32 * 32, full * sms
+    t = np.arange(n * rows) + 0.1
+    y = np.random.default_rng(3).standard_normal(n * rows).astype(np.float32)
+    theta = torch.tensor([THETA[(SHO,)]] * rows, dtype=torch.float32, device="cuda")
+    n_launch = []
+    for ck in (32, 16):
+        m = gp.Model((SHO,), np.arange(rows + 1) * n, t, t + 0.5, y,
+                     np.full(n * rows, 0.1, np.float32), chunk_len=64, ckpt_interval=ck)
+        assert m.info["n_chunks"] == 32 * rows
+        n_launch.append(launches(gp, lambda: m.loglik_grad(theta))[0])
+    assert n_launch[0] - n_launch[1] == (2 if parallel else 0)

@@ -23,7 +23,7 @@ def plan():
     return ctypes.CDLL(out)
 
 
-# product, combination precision, D, longest chunk, ck, chunks, SMs -> segments
+# product, combination precision, D, longest chunk, ck, chunks, SMs (, mean) -> segments
 @pytest.mark.parametrize("case,want", [
     ((0, 32, 6, 256, 32, 320, 152), 8),
     ((0, 32, 6, 33, 32, 320, 152), 2),
@@ -34,14 +34,20 @@ def plan():
     ((1, 32, 4, 256, 32, 320, 152), 1),            # product kernels have none
     ((0, 32, 6, 256, 32, 32 * 6 * 152, 152), 8),   # the line, and past it
     ((0, 32, 6, 256, 32, 32 * (6 * 152 + 1), 152), 1),
-    ((0, 32, 4, 256, 32, 32 * 12 * 152, 152), 8),
-    ((0, 32, 4, 256, 32, 32 * (12 * 152 + 1), 152), 1),
+    ((0, 32, 4, 256, 32, 32 * 7 * 152, 152), 8),   # equal chunks
+    ((0, 32, 4, 256, 32, 32 * (7 * 152 + 1), 152), 1),
+    ((0, 32, 4, 240, 32, 32 * 12 * 152, 152, 140), 8),   # 7 / 12 of the longest on average
+    ((0, 32, 4, 240, 32, 32 * 12 * 152, 152, 141), 1),
+    ((0, 32, 4, 256, 32, 32 * (12 * 152 + 1), 152, 100), 1),
+    ((0, 32, 6, 256, 32, 32 * (6 * 152 + 1), 152, 100), 1),
     ((0, 32, 6, 32 * 1024, 32, 32, 152), 1024),
     ((0, 32, 6, 32 * 1024 + 1, 32, 32, 152), 1),
     ((0, 32, 7, 1024, 32, 29184, 152), 1),         # past 2 GiB of replay
 ])
 def test_segments_of_a_gradient(plan, case, want):
-    assert plan.ph_grad_segments(*case) == want
+    # all chunks as long as the longest, or of the mean length given last
+    *args, mean = case if len(case) == 8 else (*case, case[3])
+    assert plan.ph_grad_segments(*args, ctypes.c_int64(args[5] * mean)) == want
 
 
 # bytes of the buffers: needed, of the fast way, of the plain way
