@@ -51,6 +51,10 @@ inline int grad_segments(const SegmentCase &c) {
   constexpr size_t kMaxReplay = (size_t)2 << 30;  // bytes of the replay buffers
   // shorter segments would put a boundary adjoint's rounding every few events
   if (c.product || c.comb_prec != 32 || c.ck < 32) return 1;
+  // and a second segment of less than half the events gives too little: 608 warps
+  // of chunks of 34 events 282 us against 256 in turn, of 40 290 against 275, of
+  // 48 302 against 301, of 64 323 against 353 (two SHO terms)
+  if (2 * c.max_chunk < 3 * c.ck) return 1;
   const int n_seg = (c.max_chunk + c.ck - 1) / c.ck;
   const int per_sm = c.D <= 4 ? 12 : 6;
   if (c.n_vch / 32 > per_sm * c.n_sm || n_seg < 2 || n_seg > kMaxSegments) return 1;

@@ -32,15 +32,15 @@ def launches(gp, f):
 @pytest.mark.parametrize("terms", list(THETA))
 @pytest.mark.parametrize("prec", [32, 64])
 def test_fp64_combination_walks_in_turn(terms, prec):
-    # 700 exposures: chunks of 44 events, two segments.  With the combination
+    # 1000 exposures: chunks of up to 64 events, two segments.  With the combination
     # in FP64 every segment starts from what was walked back from the FP64
     # adjoint at the chunk's end, as with segments too short for threads of
     # their own (ckpt_interval = 16).
     import paper_2601_02527_gb300 as gp
     oracle.build()
     theta = torch.tensor([THETA[terms]], dtype=torch.float32, device="cuda")
-    m, data = build(gp, terms, 700, combine_precision=prec)
-    turn, _ = build(gp, terms, 700, combine_precision=prec, ckpt_interval=16)
+    m, data = build(gp, terms, 1000, combine_precision=prec)
+    turn, _ = build(gp, terms, 1000, combine_precision=prec, ckpt_interval=16)
     n, (ll, g) = launches(gp, lambda: m.loglik_grad(theta))
     n1, _ = launches(gp, lambda: turn.loglik_grad(theta))
     assert n == n1 + (2 if prec == 32 else 0)
@@ -49,17 +49,18 @@ def test_fp64_combination_walks_in_turn(terms, prec):
     assert nc == nc1 + (2 if prec == 32 else 0)
     ref_ll, ref = oracle.loglik(list(terms), 0, *data, np.array(THETA[terms], np.float32)
                                 .astype(np.float64), grad=True)
-    assert abs(ll.item() - ref_ll) <= 1e-4 * max(abs(ref_ll), 70.0)
+    assert abs(ll.item() - ref_ll) <= 1e-4 * max(abs(ref_ll), 100.0)
     g = g[0].cpu().numpy().astype(np.float64)
     assert np.all(np.abs(g - ref) <= 1e-3 * np.abs(ref) + 1e-4 * np.abs(ref).max())
 
 
-@pytest.mark.parametrize("full,parallel", [(5, True), (8, False)])
-def test_equal_chunks_past_the_line_walk_in_turn(full, parallel):
-    # states of 3, `full` warps per SM of chunks of 64 events each
+@pytest.mark.parametrize("full,length,parallel", [(5, 64, True), (8, 64, False), (1, 48, True),
+                                                  (1, 46, False)])
+def test_equal_chunks_past_the_line_walk_in_turn(full, length, parallel):
+    # states of 3, `full` warps per SM of chunks of `length` events each
     import paper_2601_02527_gb300 as gp
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    n, rows = 32 * 32, full * sms
+    n, rows = 16 * length, full * sms
     t = np.arange(n * rows) + 0.1
     y = np.random.default_rng(3).standard_normal(n * rows).astype(np.float32)
     theta = torch.tensor([THETA[(SHO,)]] * rows, dtype=torch.float32, device="cuda")

@@ -26,7 +26,10 @@ def plan():
 # product, combination precision, D, longest chunk, ck, chunks, SMs (, mean) -> segments
 @pytest.mark.parametrize("case,want", [
     ((0, 32, 6, 256, 32, 320, 152), 8),
-    ((0, 32, 6, 33, 32, 320, 152), 2),
+    ((0, 32, 6, 48, 32, 320, 152), 2),
+    ((0, 32, 6, 47, 32, 320, 152), 1),             # a short second segment
+    ((0, 32, 6, 95, 64, 320, 152), 1),
+    ((0, 32, 6, 96, 64, 320, 152), 2),
     ((0, 32, 6, 32, 32, 320, 152), 1),             # one segment is the chunk
     ((0, 64, 6, 256, 32, 320, 152), 1),            # FP64 adjoints at chunk ends: walked on
     ((0, 64, 3, 256, 64, 320, 152), 1),
