@@ -2206,8 +2206,15 @@ cudaError_t launch_warp_combine(const DevModel &M, const float *ef, int n_vch, v
         k_warp_scan_coop<S><<<dim3(n_w, dirs), 32 * COOP, 0, st>>>(ef, n_vch, pre_local,
                                                                    suf_local, wtot);
     }
-    // a warp per series and direction until the series alone fill the GPU
-    coop_fold = n_out <= 64 * M.n_sm;
+    // a warp per series and direction where the series are few; one thread each
+    // fills its warps' lanes from some 10 series per SM on (25 for states of 7).
+    // The whole combination with the backward direction, series of one warp of
+    // chunks: states of 4, 512 series 33.1 us against 33.5, 2048 60.1 against
+    // 60.2, 9728 213 against 205; of 6, 1024 series 92 against 95, 3072 235
+    // against 231; of 7, 1024 series 184 against 194, 3072 423 against 430, 9728
+    // 1243 against 1237.  Of eight warps, states of 6: 512 series 320 against 349,
+    // 1536 870 against 879, 3072 1675 against 1664.
+    coop_fold = n_out <= (S::D < 7 ? 10 : 25) * M.n_sm;
   }
   if (!coop)
     // the two directions are independent: blocks of their own
