@@ -1084,34 +1084,34 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
                                    (int64_t)rows * m->dcache_steps, m->n_sm});
     const size_t exp_ev = (size_t)(per_series ? 1 : n_sets) * m->n_events;
     const size_t part = m->n_params * nv * sizeof(float);
-    std::vector<gpss::Buffer> needed, fast, plain;
+    std::vector<gpss::Buffer> first, rest, fast, late, plain;
     auto put = [](std::vector<gpss::Buffer> &list, auto &p, size_t bytes) {
       list.push_back({(void **)&p, bytes});
     };
-    put(needed, ef, o.NF * nv * sizeof(float));
-    put(needed, ed, o.ND * nv * sizeof(double));
-    put(needed, tabs, (size_t)n_sets * o.NT * gpss::TAB_TERM * sizeof(float));
-    if (grad || tree) put(needed, state_end, SD * nv * eb);
+    put(first, ef, o.NF * nv * sizeof(float));
+    put(first, ed, o.ND * nv * sizeof(double));
+    put(first, tabs, (size_t)n_sets * o.NT * gpss::TAB_TERM * sizeof(float));
+    if (grad || tree) put(rest, state_end, SD * nv * eb);
     if (tree) {
-      put(needed, ll_part, nv * sizeof(double));
-      put(needed, pre_local, o.NF * nv * eb);
-      put(needed, wtot, o.NF * n_w * eb);
-      put(needed, wpre, o.NF * n_w * eb);
-      put(needed, scratch, cb.warp_scratch(n_vch) * eb);
+      put(rest, ll_part, nv * sizeof(double));
+      put(rest, pre_local, o.NF * nv * eb);
+      put(rest, wtot, o.NF * n_w * eb);
+      put(rest, wpre, o.NF * n_w * eb);
+      put(rest, scratch, cb.warp_scratch(n_vch) * eb);
       if (grad) {
-        put(needed, info, SD * nv * eb);
-        put(needed, suf_local, o.NF * nv * eb);
-        put(needed, wsuf, o.NF * n_w * eb);
+        put(rest, info, SD * nv * eb);
+        put(rest, suf_local, o.NF * nv * eb);
+        put(rest, wsuf, o.NF * n_w * eb);
       }
     }
-    if (grad) put(needed, adj, SD * nv * sizeof(float));
+    if (grad) put(rest, adj, SD * nv * sizeof(float));
     if (dexp) {
-      put(needed, gdt, exp_ev * sizeof(float));
-      put(needed, gwe, exp_ev * sizeof(float));
+      put(rest, gdt, exp_ev * sizeof(float));
+      put(rest, gwe, exp_ev * sizeof(float));
     }
-    if (cond_out) put(needed, cond, exp_ev * sizeof(float2));
+    if (cond_out) put(rest, cond, exp_ev * sizeof(float2));
     if (m->product) {
-      if (grad) put(needed, gpart, part);
+      if (grad) put(rest, gpart, part);
       // the oscillators' scalars of every step (the gradient's with their
       // tangents); without them every thread forms its own step by step
       const size_t bytes = rows * (size_t)m->dcache_steps * (o.D / 2) * sizeof(float4);
@@ -1122,25 +1122,27 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
         if (grad) put(fast, ptan, 2 * bytes);
       }
     } else if (grad) {
-      put(needed, ckpt, n_pck * (o.NF + 1) * nv * sizeof(float));
+      put(first, ckpt, n_pck * (o.NF + 1) * nv * sizeof(float));
       // the element pass keeps every step's scalars for the gradient's replay
       // while that takes at most kDcacheMax bytes (else the replay recomputes them)
       const size_t bytes =
           rows * (size_t)m->dcache_steps * (4 * ((6 * o.NT + 3) / 4)) * sizeof(float);
-      if (m->step_cache == 0 && bytes <= kDcacheMax) put(needed, dcache, bytes);
+      if (m->step_cache == 0 && bytes <= kDcacheMax) put(first, dcache, bytes);
       put(plain, rbuf, gpss::replay_bytes(ck, o.D, o.NP, n_vch, 1));
       put(plain, gpart, part);
       if (n_seg > 1) {
         const size_t rec = (n_seg - 1) * nv * sizeof(float);
-        // the largest first: where a later one fails, the plain way's replay
-        // fits into what this one gives back
-        put(fast, rbuf, gpss::replay_bytes(ck, o.D, o.NP, n_vch, n_seg));
         put(fast, segel, rec * o.NF);
-        put(fast, seg_info, rec * SD);
-        put(fast, seg_adj, rec * SD);
-        put(fast, gpart, n_seg * part);
+        put(late, rbuf, gpss::replay_bytes(ck, o.D, o.NP, n_vch, n_seg));
+        put(late, seg_info, rec * SD);
+        put(late, seg_adj, rec * SD);
+        put(late, gpart, n_seg * part);
       }
     }
+    // the fast way's and the plain way's after the first kernels; the fast one's
+    // largest first, so that the plain one's fit into what it gives back
+    late.insert(late.end(), rest.begin(), rest.end());
+    plain.insert(plain.end(), rest.begin(), rest.end());
     // a capture records allocations without making them, and a graph's come in
     // larger pieces: the fast way's are recorded only if the device has twice
     // the call's memory now (free, or kept by graphs that ended)
@@ -1154,10 +1156,11 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
               cudaSuccess ||
           cudaDeviceGetGraphMemAttribute(m->device, cudaGraphMemAttrUsedMemCurrent, &used) !=
               cudaSuccess ||
-          2 * (gpss::total_bytes(needed) + gpss::total_bytes(fast)) > avail + (kept - used))
+          2 * (gpss::total_bytes(first) + gpss::total_bytes(fast) + gpss::total_bytes(late)) >
+              avail + (kept - used))
         fast.clear();
     }
-    const gpss::Scratch way = gpss::take_scratch(needed, fast, plain, take, give);
+    gpss::Scratch way = gpss::take_first(first, fast, take, give);
     if (way == gpss::Scratch::none) {
       res = GP_SS_ENOMEM;
       break;
@@ -1189,6 +1192,19 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
       }
       if (res) break;
     }
+    const bool begun = way == gpss::Scratch::fast;
+    way = gpss::take_rest(way, fast, late, plain, take, give);
+    // the pool keeps what was given back in pieces of its own; once the kernels
+    // have left them, the device has it again
+    if (way == gpss::Scratch::none && begun && m->pool &&
+        cudaStreamSynchronize(st) == cudaSuccess &&
+        cudaMemPoolTrimTo(m->pool, 0) == cudaSuccess && gpss::take_all(plain, take, give))
+      way = gpss::Scratch::plain;
+    if (way == gpss::Scratch::none) {
+      res = GP_SS_ENOMEM;
+      break;
+    }
+    if (way == gpss::Scratch::plain) n_seg = 1;
     {
       PhaseTimer pt(m, st, 1);
       cudaError_t e;

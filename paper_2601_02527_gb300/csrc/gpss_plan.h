@@ -140,15 +140,31 @@ bool take_all(const std::vector<Buffer> &list, Take take, Give give) {
 
 enum class Scratch { none, plain, fast };
 
-// A call's scratch: what both of its ways need, then the buffers of the fast
-// way or, where they cannot be had, of the plain one.  The fast way's are
-// taken last, so that a call is refused only where the plain way does not fit.
+// A call's scratch in two steps, so that the second step's allocations run
+// behind the first kernels.  First what these need, then what they need for
+// the fast way, all or none.
 template <class Take, class Give>
-Scratch take_scratch(const std::vector<Buffer> &needed, const std::vector<Buffer> &fast,
-                     const std::vector<Buffer> &plain, Take take, Give give) {
-  if (!take_all(needed, take, give)) return Scratch::none;
-  if (!fast.empty() && take_all(fast, take, give)) return Scratch::fast;
-  return take_all(plain, take, give) ? Scratch::plain : Scratch::none;
+Scratch take_first(const std::vector<Buffer> &first, const std::vector<Buffer> &fast, Take take,
+                   Give give) {
+  if (!take_all(first, take, give)) return Scratch::none;
+  return !fast.empty() && take_all(fast, take, give) ? Scratch::fast : Scratch::plain;
+}
+
+// Then the rest of either way.  Where the fast way's cannot be had, its buffers
+// of the first step are given back for the plain one's: a call is refused only
+// where the plain way does not fit.
+template <class Take, class Give>
+Scratch take_rest(Scratch way, const std::vector<Buffer> &fast,
+                  const std::vector<Buffer> &rest_fast, const std::vector<Buffer> &rest_plain,
+                  Take take, Give give) {
+  if (way == Scratch::fast) {
+    if (take_all(rest_fast, take, give)) return Scratch::fast;
+    for (const Buffer &b : fast) {
+      give();
+      *b.p = nullptr;
+    }
+  }
+  return take_all(rest_plain, take, give) ? Scratch::plain : Scratch::none;
 }
 
 }  // namespace gpss

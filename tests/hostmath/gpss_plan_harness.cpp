@@ -23,13 +23,15 @@ int ph_upload_groups(const int64_t *ev_off, const int32_t *ch_first, int n_serie
   return (int)c.size() - 1;
 }
 
-// take_scratch against an allocator of `limit` bytes.  n[3], bytes: the lists
-// (needed, fast, plain) one after the other; held: bytes taken in the end;
-// got[i]: buffer i is in hand.  Returns 0 none, 1 plain, 2 fast.
-int ph_take_scratch(size_t limit, const int *n, const size_t *bytes, size_t *held, int *got) {
-  std::vector<void *> addr(n[0] + n[1] + n[2], (void *)8);
-  std::vector<Buffer> list[3];
-  for (int l = 0, i = 0; l < 3; ++l)
+// take_first and take_rest against an allocator of `limit` bytes.  n[4], bytes:
+// the lists (first, fast, and the rest of the fast and of the plain way); held: bytes taken
+// in the end; got[i]: buffer i is in hand; begun: the way after the first step.
+// Returns 0 none, 1 plain, 2 fast.
+int ph_take_scratch(size_t limit, const int *n, const size_t *bytes, size_t *held, int *got,
+                    int *begun) {
+  std::vector<void *> addr(n[0] + n[1] + n[2] + n[3], (void *)8);
+  std::vector<Buffer> list[4];
+  for (int l = 0, i = 0; l < 4; ++l)
     for (int k = 0; k < n[l]; ++k, ++i) list[l].push_back({&addr[i], bytes[i]});
   std::vector<size_t> taken;
   *held = 0;
@@ -44,7 +46,9 @@ int ph_take_scratch(size_t limit, const int *n, const size_t *bytes, size_t *hel
     *held -= taken.back();
     taken.pop_back();
   };
-  const Scratch way = take_scratch(list[0], list[1], list[2], take, give);
+  Scratch way = take_first(list[0], list[1], take, give);
+  *begun = way == Scratch::none ? 0 : way == Scratch::plain ? 1 : 2;
+  if (way != Scratch::none) way = take_rest(way, list[1], list[2], list[3], take, give);
   for (size_t i = 0; i < addr.size(); ++i) got[i] = addr[i] != nullptr;
   return way == Scratch::none ? 0 : way == Scratch::plain ? 1 : 2;
 }

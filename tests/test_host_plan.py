@@ -53,30 +53,34 @@ def test_segments_of_a_gradient(plan, case, want):
     assert plan.ph_grad_segments(*args, ctypes.c_int64(args[5] * mean)) == want
 
 
-# bytes of the buffers: needed, of the fast way, of the plain way
-@pytest.mark.parametrize("needed,fast,plain", [
-    ([100, 40, 16], [800, 70, 30], [100, 16]),     # segments of a gradient
-    ([100, 40, 16], [300, 600], []),               # a product model's scalars
-    ([100, 40, 16], [], [50]),
-    ([100], [64], [64]),
+# bytes of the buffers: of the first kernels, theirs of the fast way, the rest
+# of the fast and of the plain way
+@pytest.mark.parametrize("first,fast,late,plain", [
+    ([100, 40, 16], [70], [800, 30, 60, 20], [100, 16, 60, 20]),   # segments of a gradient
+    ([100, 40, 16], [300, 600], [70], [70]),                       # a product model's scalars
+    ([100, 40], [], [], [50, 16, 30]),
+    ([100], [64], [500], [564]),
 ])
-def test_scratch_is_refused_only_where_the_plain_way_does_not_fit(plan, needed, fast, plain):
-    lists = [needed, fast, plain]
-    n = (ctypes.c_int * 3)(*[len(x) for x in lists])
+def test_scratch_is_refused_only_where_the_plain_way_does_not_fit(plan, first, fast, late, plain):
+    lists = [first, fast, late, plain]
+    n = (ctypes.c_int * 4)(*[len(x) for x in lists])
     flat = sum(lists, [])
     size = (ctypes.c_size_t * len(flat))(*flat)
-    for limit in range(sum(needed) + sum(fast) + sum(plain) + 2):
-        held, got = ctypes.c_size_t(), (ctypes.c_int * len(flat))()
-        way = plan.ph_take_scratch(ctypes.c_size_t(limit), n, size, ctypes.byref(held), got)
-        with_fast, with_plain = sum(needed) + sum(fast), sum(needed) + sum(plain)
-        want = 2 if fast and with_fast <= limit else int(with_plain <= limit)
-        assert way == want, (limit, way)
+    for limit in range(sum(flat) + 2):
+        held, got, begun = ctypes.c_size_t(), (ctypes.c_int * len(flat))(), ctypes.c_int()
+        way = plan.ph_take_scratch(ctypes.c_size_t(limit), n, size, ctypes.byref(held), got,
+                                   ctypes.byref(begun))
+        with_fast, with_plain = sum(first + fast + late), sum(first + plain)
+        assert way == (2 if fast and with_fast <= limit else int(with_plain <= limit)), limit
+        assert begun.value == (2 if fast and sum(first + fast) <= limit else
+                               int(sum(first) <= limit))
+        hand = [list(got)[i:i + len(x)] for i, x in
+                zip(np.cumsum([0, *map(len, lists)]), lists)]
         if way == 2:
-            assert held.value == with_fast and all(got[:len(needed) + len(fast)])
+            assert held.value == with_fast and all(sum(hand[:3], []))
         elif way == 1:
-            assert held.value == with_plain
-            assert list(got)[:len(flat) - len(plain)] == [1] * len(needed) + [0] * len(fast)
-            assert all(list(got)[len(flat) - len(plain):])
+            assert held.value == with_plain and all(hand[0] + hand[3])
+            assert not any(hand[1])
 
 
 FULL = 152 * 128  # chunks of one block per multiprocessor
