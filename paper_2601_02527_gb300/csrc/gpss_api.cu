@@ -1149,15 +1149,17 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (!fast.empty() && cudaStreamIsCapturing(st, &cs) == cudaSuccess &&
         cs != cudaStreamCaptureStatusNone) {
+      const size_t twice = 2 * (gpss::total_bytes(first) + gpss::total_bytes(fast) +
+                                gpss::total_bytes(late));
       size_t avail = 0, total = 0;
       uint64_t kept = 0, used = 0;
       if (cudaMemGetInfo(&avail, &total) != cudaSuccess ||
-          cudaDeviceGetGraphMemAttribute(m->device, cudaGraphMemAttrReservedMemCurrent, &kept) !=
-              cudaSuccess ||
-          cudaDeviceGetGraphMemAttribute(m->device, cudaGraphMemAttrUsedMemCurrent, &used) !=
-              cudaSuccess ||
-          2 * (gpss::total_bytes(first) + gpss::total_bytes(fast) + gpss::total_bytes(late)) >
-              avail + (kept - used))
+          (twice > avail &&
+           (cudaDeviceGetGraphMemAttribute(m->device, cudaGraphMemAttrReservedMemCurrent, &kept) !=
+                cudaSuccess ||
+            cudaDeviceGetGraphMemAttribute(m->device, cudaGraphMemAttrUsedMemCurrent, &used) !=
+                cudaSuccess ||
+            twice > avail + (kept - used))))
         fast.clear();
     }
     gpss::Scratch way = gpss::take_first(first, fast, take, give);
