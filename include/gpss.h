@@ -28,6 +28,18 @@
  *  - Scratch memory is taken from the stream-ordered allocator
  *    (cudaMallocAsync) on the caller's stream and released before the call
  *    returns, so calls on different streams may share one model.
+ *    A model's pool keeps what its largest call took until the model is freed.
+ *    Gradients and conditioned values of few chunks take up to about 2.5 GB
+ *    more to walk a chunk's segments in parallel, product kernels up to 8 GB
+ *    for step scalars (step_cache); where the memory is not there the call
+ *    runs without, more slowly.  A call recorded in a stream capture takes
+ *    them only if the device has twice the call's memory free at that time.
+ *  - Rounding: a row's gradient and conditioned values may differ in their
+ *    last FP32 digits with the number of chunks in the call (the other series,
+ *    the parameter sets, a shard of the batch) and with the memory free,
+ *    because these decide between parallel segments and segments in turn.  The
+ *    log-likelihood of a series depends on the rest of the call only through
+ *    whether some series has more than 512 chunks (another combination tree).
  *  - Hyperparameters are natural parameters, one row of n_params floats per
  *    set: per term (sigma, omega0, Q) for GP_SS_TERM_SHO (any Q > 0: the
  *    overdamped oscillator Q < 1/2 of Appendix B included), (sigma, ell)
@@ -108,16 +120,21 @@ typedef struct {
                              1 sequential fold per series (one thread per series),
                              2 parallel scan (Section 3.2.5): each warp's 32 chunks in
                                shared memory, then a tree scan of the warp totals */
-  int step_cache;         /* gradient calls: 0 auto -- the element pass keeps every step's
-                             per-term scalars (f, f', F1, I_ff, I_pp, I_FF) in device
-                             memory for the reverse sweep while they take at most 8 GiB
-                             (24 bytes per event and term per theta set), else the sweep
-                             recomputes them; 1 always recompute */
+  int step_cache;         /* per-step scalars kept in device memory: 0 auto, while they take
+                             at most 8 GiB; 1 never.  Gradient calls keep those the element
+                             pass forms for the reverse sweep (f, f', F1, I_ff, I_pp, I_FF:
+                             24 bytes per event and term per theta set), else the sweep
+                             recomputes them.  Product kernels form f, f', I_ff, I_pp for
+                             all steps first (16 bytes per event and oscillator, 48 with
+                             their tangents for a gradient; log-likelihood calls only where
+                             chunks are long and few), else step by step. */
   int combine_precision;  /* arithmetic of the combination of chunk elements across a series
                              (every level of the scan of Section 3.2.5, the closed-form chunk
                              log-likelihoods and the adjoints at chunk ends): 0 auto (= 32),
-                             64 FP64, 32 FP32.  The chunk elements themselves are always
-                             FP32; the log-likelihood sums are always FP64. */
+                             64 FP64 (gradient segments are then walked in turn from the
+                             FP64 adjoint at the chunk's end), 32 FP32.  The chunk elements
+                             themselves are always FP32; the log-likelihood sums are always
+                             FP64. */
 } gp_ss_options;
 
 /* Build a model from exposures (Section 3.2: two events per exposure, reset
@@ -218,10 +235,10 @@ gp_ss_status gp_ss_loglik_grad_batched(const gp_ss_model *model, const float *th
  * (host f32) to the device, optionally re-uploads the model's event stream
  * from its pinned host copy (reupload_events != 0), computes, and copies the
  * results back into host buffers before returning (synchronous).  The
- * re-upload goes in series groups on an internal copy stream (it first waits
- * for the work already queued on cuda_stream), each group's element pass
- * starting once its events are in; it rewrites the model's device copy, so
- * it must not run concurrently with other calls on the same model. */
+ * re-upload goes in up to four series groups on an internal copy stream (it
+ * first waits for the work already queued on cuda_stream), each group's
+ * element pass starting once its events are in; it rewrites the model's device
+ * copy, so it must not run concurrently with other calls on the same model. */
 gp_ss_status gp_ss_loglik_grad_host(const gp_ss_model *model, const float *theta_host,
                                     int n_sets, int theta_per_series, double *loglik_host,
                                     float *grad_host, int reupload_events, void *cuda_stream);

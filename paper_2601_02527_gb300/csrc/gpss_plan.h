@@ -40,12 +40,14 @@ inline size_t replay_bytes(int ck, int D, int NP, int n_vch, int n_seg) {
 // warps of instants took 995 us against 1145 (1195 against 1214), SHO alone 561
 // against 617 (639 against 659).  So: up to 6 warps of chunks per SM, or for
 // states of at most 4 up to 12 that have no more steps than 7 of the longest.
-// The adjoint at a segment's end differs from the walked one in rounding;
-// exposure gradients and predictions, differences of nearly equal terms, would
-// show it at 3e-5 of their size and keep the walk in turn.  The segments'
-// elements and the information carried back through them are FP32: a model
-// whose combination runs in FP64 starts the walk in turn from the FP64 adjoint
-// at the chunk's end and keeps it.
+// The adjoint at a segment's end differs from the walked one in rounding, which
+// shows in differences of nearly equal terms: with parallel segments, 1600
+// exposures of one SHO term, the exposure gradient's error against FP64 is 5.7e-6
+// of its largest instead of 3.9e-6 and a predicted variance's 1.0e-4 instead of
+// 6.1e-5.  Exposure gradients and predictions keep the walk in turn.  The
+// segments' elements and the information carried back through them are FP32: a
+// model whose combination runs in FP64 starts the walk in turn from the FP64
+// adjoint at the chunk's end and keeps it.
 inline int grad_segments(const SegmentCase &c) {
   constexpr int kMaxSegments = 1024;  // k_seg_info carries the adjoints back through them in turn
   constexpr size_t kMaxReplay = (size_t)2 << 30;  // bytes of the replay buffers
@@ -65,7 +67,7 @@ inline int grad_segments(const SegmentCase &c) {
 // Whether a product model's step scalars are formed for all steps at once
 // rather than by the chunks' threads.  For a gradient always: every
 // parameter's thread reads them (150 series of 500 to 5000 instants 1633 ->
-// 642 us; one of 100: 92 -> 86 us).  The log-likelihood alone reads each once:
+// 601 us; one of 100: 92 -> 86 us).  The log-likelihood alone reads each once:
 // they shorten a chunk's serial chain but cost a pass over memory and two
 // launches, so they are formed where chunks are long and warps of chunks too
 // few to hide the chain.  Product alone (two oscillators), at once against

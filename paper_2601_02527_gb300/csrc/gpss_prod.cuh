@@ -72,7 +72,7 @@ GPSS_HD Osc2<T> osc2(F dt, T w0, T Q, T var) {
 // l of warp w at ((w_doff[w] + 32 k) NO + 32 j + l); with tangents, two more
 // float4 (s d/da, s^2 d/dbeta of the four, s = prod_unit) in an array of their
 // own, in the same order.  150 series of 500 to 5000 instants with the gradient, product +
-// Matern-3/2: scalars 67 us, elements 442 -> 121 us, gradient 1099 -> 304 us.
+// Matern-3/2: scalars 67 us, elements 442 -> 121 us, gradient 1099 -> 324 us.
 // ---------------------------------------------------------------------------
 template <bool SUM>
 struct ProdOsc {
