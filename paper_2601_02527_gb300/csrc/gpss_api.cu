@@ -1199,7 +1199,7 @@ gp_ss_status enqueue(const gp_ss_model *m, const float *theta, int n_sets, int p
     // the pool keeps what was given back in pieces of its own; once the kernels
     // have left them, the device has it again
     if (way == gpss::Scratch::none && begun && m->pool &&
-        cudaStreamSynchronize(st) == cudaSuccess &&
+        cs == cudaStreamCaptureStatusNone && cudaStreamSynchronize(st) == cudaSuccess &&
         cudaMemPoolTrimTo(m->pool, 0) == cudaSuccess && gpss::take_all(plain, take, give))
       way = gpss::Scratch::plain;
     if (way == gpss::Scratch::none) {
